@@ -84,7 +84,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(),
 # The sources the streaming step kernel is compiled from (its DRAM traffic
 # recorded under profiles/ stays valid while they are unchanged; the public
 # header contributes only enum constants to it).
-STEP_KERNEL_SOURCES = (os.path.join(CSRC, "fk_stream.cu"), os.path.join(CSRC, "fk_internal.cuh"))
+STEP_KERNEL_SOURCES = (os.path.join(CSRC, "fk_stream.cu"),
+                       os.path.join(CSRC, "fk_stream_unit.cuh"),
+                       os.path.join(CSRC, "fk_internal.cuh"))
 
 
 def code_only(text: str) -> str:

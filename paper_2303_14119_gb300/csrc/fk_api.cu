@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "fk_host.cuh"
+#include "fk_resident.cuh"
 
 using namespace fk;
 
@@ -23,6 +24,10 @@ namespace {
 thread_local std::string g_create_error;
 
 constexpr int kGraphSteps = 32;  // steps per captured graph (even)
+// what the re-emission in a resident launch's first chunk and the boundary
+// sums in its last one cost, in planes (5 and 7 us a launch-step against 1.5
+// us a plane at 321 x 117 x 117; more than 2 left the other chunks too long)
+constexpr int kResidentFirst = 2, kResidentLast = 2;
 constexpr int kMaxTimed = 8192;  // step-kernel launches timed between reads
 constexpr size_t kStageElems = size_t(1) << 23;  // FP64 staging chunk, 64 MB
 
@@ -162,10 +167,14 @@ fk_status fk::replan_tiles(fk_grid* g, int cap) {
   const Geom old_geom = g->geom;
   const int old_cap = g->tile_cap;
   const bool old_stream = g->use_stream;
+  const int old_len = g->res_chunk_len, old_off = g->res_chunk_off, old_chunks = g->res_chunks;
   auto restore = [&](fk_status s) {
     g->geom = old_geom;
     g->tile_cap = old_cap;
     g->use_stream = old_stream;
+    g->res_chunk_len = old_len;
+    g->res_chunk_off = old_off;
+    g->res_chunks = old_chunks;
     return s;
   };
   g->tile_cap = cap;
@@ -175,9 +184,10 @@ fk_status fk::replan_tiles(fk_grid* g, int cap) {
   const int nu = g->geom.n_tiles;
   if (nu > g->part_cap) {  // more tiles: larger partial-sum buffers (the grid is idle)
     const size_t nparts = (size_t)g->nx * nu;
-    const size_t sizes[5] = {nparts, nparts, (size_t)nu, (size_t)nu, (size_t)nu};
-    double* nb[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    for (int q = 0; q < 5; q++) {
+    constexpr int kBufs = 6;
+    const size_t sizes[kBufs] = {nparts, nparts, nparts, (size_t)nu, (size_t)nu, (size_t)nu};
+    double* nb[kBufs] = {};
+    for (int q = 0; q < kBufs; q++) {
       cudaError_t e = hooked_alloc(reinterpret_cast<void**>(&nb[q]), sizes[q] * sizeof(double));
       if (e == cudaSuccess) e = cudaMemsetAsync(nb[q], 0, sizes[q] * sizeof(double), g->stream);
       if (e != cudaSuccess) {
@@ -191,8 +201,9 @@ fk_status fk::replan_tiles(fk_grid* g, int cap) {
       for (double* p : nb) cudaFree(p);
       return restore(cuda_fail(g, e, "cudaStreamSynchronize"));
     }
-    double** bufs[5] = {&g->part.n, &g->part.lv, &g->part.pe, &g->part.see, &g->part.vac};
-    for (int q = 0; q < 5; q++) {
+    double** bufs[kBufs] = {&g->part.n,  &g->part.lv,  &g->d_lv_odd,
+                            &g->part.pe, &g->part.see, &g->part.vac};
+    for (int q = 0; q < kBufs; q++) {
       if (*bufs[q]) cudaFree(*bufs[q]);
       *bufs[q] = nb[q];
     }
@@ -292,6 +303,15 @@ cudaError_t enqueue_step(fk_grid* g, int cur, cudaStream_t s, cudaEvent_t ev0, c
   return e;
 }
 
+// Whether fk_step runs on the resident step kernel: the unsplit scheme on
+// streaming tiles, at every size (it was the faster one from 64 x 48 x 48 to
+// 1024 x 256 x 256, in both storage types; figures in fk_resident.cu).  (A withheld pipeline item, a test knob, has to lie in the
+// first step of the unit it names.)
+bool use_resident(const fk_grid* g) {
+  return g->use_stream && g->scheme == kSchemeUnsplit && g->res_chunks > 0 &&
+         g->prm.withhold_item < g->res_chunk_len - g->res_chunk_off;
+}
+
 // Calls that change a grid's state are refused while a batch steps it.
 #define FK_NOT_IN_BATCH(g)                                                          \
   do {                                                                              \
@@ -353,9 +373,9 @@ void free_grid(fk_grid* g) {
   void* ptrs[] = {g->d_prm, g->d_st, g->d_f[0], g->d_f[1], g->tab.v1, g->tab.cx,
                   g->tab.cx32, g->tab.delta, g->tab.gse, g->tab.src, g->tab.src32,
                   g->tab.gfe_raw, g->tab.srow32, g->tab.scol32, g->tab.tsum, g->tab.m1, g->tab.m2,
-                  g->tab.m1_32, g->tab.m2_32, g->tab.v1p, g->tab.deltap,
+                  g->tab.m1_32, g->tab.m2_32, g->tab.v1p, g->tab.deltap, g->tab.vdelta,
                   g->d_bgk, g->d_bgk32, g->part.n, g->part.lv,
-                  g->part.pe, g->part.see,
+                  g->part.pe, g->part.see, g->d_res, g->d_lv_odd,
                   g->part.vac, g->d_ne, g->d_Ex, g->d_c1, g->d_c1_32, g->d_hist,
                   g->d_stage, g->d_f3, g->d_st_mid, g->d_prm_x, g->d_zero, g->d_cx_half,
                   g->d_cx32_half, g->d_lv_aside, g->fin.pre, g->fin.bsum, g->fin.blv,
@@ -424,6 +444,25 @@ fk_status build_graph(fk_grid* g, int parity) {
   return FK_OK;
 }
 
+// x-chunks of the resident step kernel: one unit per CTA, as many units as
+// fit the GPU at once beside the launch's finalize CTAs.
+void plan_resident(fk_grid* g, int sms) {
+  g->res_chunks = g->res_chunk_len = 0;
+  if (!g->use_stream) return;
+  const int per_sm = resident_ctas_per_sm(g->prec, g->geom, g->pitch, g->pitch != g->nv2);
+  const int slots = sms * per_sm - finalize_blocks(g->nx);
+  const int nc = std::min(slots / g->geom.n_tiles, g->nx);
+  if (nc < 1) return;
+  // planes that the re-emission of the first chunk and the wall and vacuum
+  // sums of the last one are worth, where chunks have planes to spare
+  const int len1 = (g->nx + nc - 1) / nc;
+  const int first = std::min(kResidentFirst, len1 - 1), last = std::min(kResidentLast, len1 - 1);
+  const int len = (g->nx + first + last + nc - 1) / nc;
+  g->res_chunk_len = len;
+  g->res_chunk_off = first;
+  g->res_chunks = (g->nx + g->res_chunk_off + len - 1) / len;
+}
+
 // Tiles of v1 rows (never straddling the sign change of v1) and chunks of
 // x-planes: one streaming unit per (tile, chunk), about one wave of them.
 // Where each sign half of the v1 rows fits the tile of a half-CTA unit,
@@ -488,6 +527,7 @@ fk_status plan_geometry(fk_grid* g) {
       m.n_chunks = (g->nx + m.chunk_len - 1) / m.chunk_len;
     }
   }
+  plan_resident(g, sms);
   return FK_OK;
 }
 
@@ -622,12 +662,15 @@ fk_status fk_create_grid(const fk_grid_desc* desc, void* cuda_stream, fk_grid** 
   CREATE_CUDA(dalloc(&g->tab.m2_32, g->pitch * sizeof(float)));
   CREATE_CUDA(dalloc(&g->tab.v1p, d.nv1 * sizeof(float2)));
   CREATE_CUDA(dalloc(&g->tab.deltap, nv * sizeof(float2)));
+  CREATE_CUDA(dalloc(&g->tab.vdelta, nv * sizeof(double)));
   CREATE_CUDA(dalloc(&g->d_bgk, 2 * (size_t)d.nx * sizeof(double)));
   CREATE_CUDA(dalloc(&g->d_bgk32, 2 * (size_t)d.nx * sizeof(float)));
   CREATE_CUDA(cudaMemsetAsync(g->d_bgk, 0, 2 * (size_t)d.nx * sizeof(double), g->stream));
   CREATE_CUDA(cudaMemsetAsync(g->d_bgk32, 0, 2 * (size_t)d.nx * sizeof(float), g->stream));
   CREATE_CUDA(dalloc(&g->part.n, nparts * sizeof(double)));
   CREATE_CUDA(dalloc(&g->part.lv, nparts * sizeof(double)));
+  CREATE_CUDA(dalloc(&g->d_lv_odd, nparts * sizeof(double)));
+  CREATE_CUDA(dalloc(&g->d_res, resident_scratch_words() * sizeof(unsigned)));
   CREATE_CUDA(dalloc(&g->part.pe, g->part.nu * sizeof(double)));
   CREATE_CUDA(dalloc(&g->part.see, g->part.nu * sizeof(double)));
   CREATE_CUDA(dalloc(&g->part.vac, g->part.nu * sizeof(double)));
@@ -844,6 +887,23 @@ fk_status fk_step(fk_grid* g, int64_t n) {
       if (rec) g->ev_used++;
       g->enq_cur ^= 1;
       n -= 1;
+    } else if (use_resident(g)) {
+      const int m = (int)std::min<int64_t>(n, kResidentSteps);
+      StepArgs a = make_args(g, g->enq_cur);
+      a.geom.chunk_len = g->res_chunk_len;
+      a.geom.n_chunks = g->res_chunks;
+      a.geom.chunk_off = g->res_chunk_off;
+      const FinOut o{g->d_ne, g->d_Ex, g->d_c1, g->d_c1_32, g->d_hist, g->fin};
+      const cudaError_t e = launch_resident(a, o, g->prec, g->prm.collisions != 0, m, g->d_lv_odd,
+                                            g->d_res, g->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {  // part of the GPU is not ours: step by step
+        cudaGetLastError();
+        g->res_chunks = 0;
+        continue;
+      }
+      FK_CUDA(g, e);
+      g->enq_cur ^= m & 1;
+      n -= m;
     } else if (n >= kGraphSteps) {
       if (!g->graph[g->enq_cur]) {
         fk_status s = build_graph(g, g->enq_cur);

@@ -31,6 +31,11 @@ struct fk_grid {
   fk::Geom geom{};
   int tile_cap = 0;   // whole-CTA v1 tiles of at most this many rows (0: the plan's most)
   int env_direct = -1, env_no_half = -1;  // FK_STEP_KERNEL / FK_STREAM_HALF at creation
+  // resident step kernel: x-chunks of its units (0 chunks: this grid does not
+  // use it), its counters and the velocity-edge partials of its odd steps
+  int res_chunk_len = 0, res_chunk_off = 0, res_chunks = 0;
+  unsigned* d_res = nullptr;
+  double* d_lv_odd = nullptr;
   int part_cap = 0;   // tiles the partial-sum buffers hold
   bool use_stream = true;  // streaming kernel (else the direct-load kernel)
   double *d_ne = nullptr, *d_Ex = nullptr, *d_c1 = nullptr, *d_hist = nullptr;

@@ -91,6 +91,7 @@ struct Tables {
   double* cx;     // [nv1] signed x-Courant numbers v1 dt / dx
   float* cx32;    // [nv1] the same rounded to FP32
   double* delta;  // [nv1][pitch] SEE yield, zero where v1 >= 0
+  double* vdelta; // [nv1][pitch] -v1 delta
   double* gse;    // [nv1][pitch] emission shape, unit flux
   double* src;    // [nv1][pitch] dt (J/e)/W g_fe, added on source planes
   float* src32;   // same rounded to FP32
@@ -126,6 +127,7 @@ struct Geom {
   int chunk_len, n_chunks;
   int stage_elems;     // elements of one shared-memory stage
   int half;            // 1: units run two to a CTA, one per half (thin tiles)
+  int chunk_off;       // resident launches: the first chunk is this much shorter
 };
 
 __host__ __device__ inline void tile_rows(const Geom& g, int nv1, int t, int* i0, int* i1,

@@ -1,0 +1,159 @@
+"""The resident step kernel (many steps of a grid in one cooperative launch)
+against the streaming kernel and the finalize kernel launched step by step.
+
+Both run the same unit code and sum in the same order, so the states, the
+moments, the history and the ledger have to be equal bit for bit, whatever
+the launch boundaries: at one plane per unit and at several, with padded
+rows, one and several finalize blocks, collisions and reflection, and with an
+E_x that changes its sign along x and in time (the planes fetched ahead of a
+step were then laid out for the other v1 neighbour)."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from oracle import QE
+from paper_2303_14119_gb300 import fk
+
+from test_gpu_parity import make_pair, rel_l1, strong_physics
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    fk.load()
+
+
+def assert_same(a, b):
+    assert np.array_equal(a.get_f(), b.get_f())
+    for x, y in zip(a.moments(), b.moments()):
+        assert np.array_equal(x, y)
+    assert a.surface_charge() == b.surface_charge()
+    assert a.ledger() == b.ledger()
+    assert a.step_count() == b.step_count()
+    n = a.step_count()[0] + 1
+    assert np.array_equal(a.history(n), b.history(n))
+
+
+# thin tiles of one plane, several planes, padded rows, one and more
+# finalize blocks (128 planes each), whole-CTA tiles
+SHAPES = [(2, 6, 5), (40, 48, 48), (131, 24, 30), (300, 40, 45), (128, 96, 72), (417, 117, 61),
+          (9, 3, 1000), (260, 256, 256)]
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("terms", [False, True])
+def test_resident_steps_equal_single_launches_bitwise(prec, shape, terms):
+    pair = []
+    for _ in range(2):
+        g, o = make_pair(shape, prec=prec)
+        f0, sigma = strong_physics(g, o, shape, seed=7, c1f=0.08)
+        if terms:  # ln Lambda such that dt nu_ee is a few percent
+            info = g.info()
+            n_max = (f0.sum(axis=(1, 2)) * info["dv1"] * info["dv2"]).max()
+            g.set_collisions(2.0, 0.03 / (info["dt"] * oracle.nu_ee(n_max, 2.0, 1.0)), True)
+            g.set_reflection(0.3)
+        g.set_state(f0, sigma)
+        pair.append(g)
+    a, b = pair
+    b.set_kernel_timing(True)  # every step: the streaming kernel, then the finalize kernel
+    for n in (1, 2, 131):  # 131: more than one launch
+        a.step(n)
+        b.step(n)
+        a.sync()
+        b.sync()
+        assert_same(a, b)
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+def test_field_changing_its_sign_between_steps(prec):
+    """The surface charge falls (no secondaries) until E_x at the wall turns
+    over, one plane after the other: their c_1 change sign within a launch."""
+    shape = (24, 40, 36)
+    pair = []
+    for _ in range(2):
+        g, o = make_pair(shape, prec=prec)
+        strong_physics(g, o, shape, seed=9)
+        g.set_see(0.0, 400.0, 1.0, 2.0, False)
+        f0 = np.full(shape, 1e5)
+        g.set_f(f0)
+        # in units of E_x's fall over one plane: E_x = 2 - (k + 1/2) at the start
+        g.set_surface_charge(4 * QE * g.info()["dx"] * g.moments()[0][0])
+        pair.append(g)
+    a, b = pair
+    b.set_kernel_timing(True)
+    a.step(120)
+    b.step(120)
+    a.sync()
+    b.sync()
+    ex = a.history(121)[:, 7]
+    assert ex[0] > 0 > ex[-1]
+    assert_same(a, b)
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+@pytest.mark.parametrize("shape", [(64, 24, 20), (200, 96, 72)])
+def test_wait_that_runs_out_ends_the_launch(prec, shape):
+    """The first item's copy withheld: every unit and finalize CTA leaves,
+    the state stays, and the GPU steps on afterwards."""
+    os.environ["FK_TEST_WAIT_CYCLES"] = "2000000"  # about 1 ms
+    os.environ["FK_TEST_WITHHOLD_COPY"] = "0"
+    try:
+        g, o = make_pair(shape, prec=prec)
+    finally:
+        del os.environ["FK_TEST_WAIT_CYCLES"]
+        del os.environ["FK_TEST_WITHHOLD_COPY"]
+    f0, sigma = strong_physics(g, o, shape, seed=31, c1f=0.05)
+    g.set_state(f0, sigma)
+    start = g.get_f()
+    assert fk.fk_step_status(g.h, 40) == fk.FK_OK  # enqueued
+    assert fk.fk_sync_status(g.h) == fk.FK_ETIMEOUT
+    out = np.empty(shape)
+    with pytest.raises(fk.FkError):
+        g.get_f(out)
+    assert np.array_equal(out, start)
+    g.close()
+    g, o = make_pair(shape, prec=prec)
+    f0, sigma = strong_physics(g, o, shape, seed=31, c1f=0.05)
+    g.set_state(f0, sigma)
+    o.set_state(g.get_f(), sigma)
+    g.step(2)
+    o.step(2)
+    assert rel_l1(g.get_f(), o.get_f()) <= (2e-12 if prec == fk.FK_F64 else 6e-7)
+    g.close()
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+def test_courant_bound_freezes_at_the_same_step(prec):
+    """A field that grows past the Courant bound during a launch: both forms
+    stop at the same state."""
+    shape = (60, 32, 28)
+    pair = []
+    for _ in range(2):
+        g, o = make_pair(shape, prec=prec)
+        f0, sigma = strong_physics(g, o, shape, seed=11)
+        g.set_source(5e11, 0.0, 1.0, 300.0)  # charges the gap until |c_1| is too large
+        g.set_state(f0, sigma)
+        pair.append(g)
+    a, b = pair
+    b.set_kernel_timing(True)
+    for g in pair:
+        g.step(400)
+        assert fk.fk_sync_status(g.h) == fk.FK_ECFL
+    fa, fb = np.empty(shape), np.empty(shape)
+    for g, f in ((a, fa), (b, fb)):
+        with pytest.raises(fk.FkError):
+            g.get_f(f)
+    assert np.array_equal(fa, fb)
+    for g in pair:
+        g.close()
