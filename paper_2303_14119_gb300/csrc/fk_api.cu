@@ -223,7 +223,7 @@ namespace {
 // Evaluate the current state: moments of f, then finalize in `mode`.
 fk_status evaluate(fk_grid* g, int mode) {
   StepArgs a = make_args(g, g->enq_cur);
-  FK_CUDA(g, launch_step(a, g->prec, 1, g->stream));
+  FK_CUDA(g, launch_moments(a, g->prec, g->stream));
   FK_CUDA(g, launch_finalize(a, g->d_ne, g->d_Ex, g->d_c1, g->d_c1_32, g->d_hist, g->fin, mode,
                              g->stream));
   return FK_OK;
@@ -293,7 +293,7 @@ cudaError_t enqueue_step(fk_grid* g, int cur, cudaStream_t s, cudaEvent_t ev0, c
       if (e == cudaSuccess) e = launch_step_pass(x2, g->prec, kPassXHalfLast, s);
     } else {
       e = g->use_stream ? launch_step_stream(a, g->prec, g->prm.collisions != 0, s)
-                        : launch_step(a, g->prec, 0, s);
+                        : launch_step(a, g->prec, s);
     }
   }
   if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, s);

@@ -92,14 +92,13 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-// Passes of the direct-load step kernel: a whole step, the moments of f_in
-// only, and the passes of the split steps: x-advection with the wall and
+// Passes of the direct-load step kernel: a whole step,
+// and the passes of the split steps: x-advection with the wall and
 // vacuum boundaries (over dt; over dt/2 without partial sums; over dt/2
 // writing every partial sum but the velocity-edge loss, the last pass of a
 // Strang step), and v1, v2 advection, source and collisions.
 enum StepPass {
   kPassFull = 0,
-  kPassMoments = 1,
   kPassX = 2,
   kPassV = 3,
   kPassXHalf = 4,

@@ -194,8 +194,10 @@ cudaError_t launch_tables(const Tables& t, int nv1, int nv2, int pitch,
                           double k_s, double T_se, double T_fe, double J_over_eW,
                           double T_e, cudaStream_t s);
 int tables_scratch_doubles();
-// Direct-load step (and moments-only evaluation): one block per (plane, tile).
-cudaError_t launch_step(const StepArgs& a, int precision, int moments_only, cudaStream_t s);
+// Direct-load step: one block per (plane, tile).
+cudaError_t launch_step(const StepArgs& a, int precision, cudaStream_t s);
+// The partial sums of a state (f_in) and its check for negative values.
+cudaError_t launch_moments(const StepArgs& a, int precision, cudaStream_t s);
 // Streaming step: one CTA per (tile, chunk), bulk-async staged planes.
 cudaError_t launch_step_stream(const StepArgs& a, int precision, bool bgk, cudaStream_t s);
 // Rows per tile of the streaming kernel for this precision and row pitch

@@ -7,6 +7,7 @@
 
 #include "fk_finalize.cuh"
 #include "fk_host.cuh"
+#include "fk_sum.cuh"
 
 namespace fk {
 
@@ -217,8 +218,8 @@ cudaError_t launch_tables(const Tables& t, int nv1, int nv2, int pitch, double v
 // ---------------------------------------------------------------------------
 // Direct-load step kernel.  One block per (plane k, tile t): the tile's rows
 // [i0, i1) times all v2 cells.  Every neighbour is a plain load (L1/L2 catch
-// the re-reads).  Used for the moments-only evaluation of a state and as the
-// step for grids whose rows do not fit the streaming kernel's tiles.
+// the re-reads).  The step of grids whose rows do not fit the streaming
+// kernel's tiles.
 //
 // Per cell, with c_x = v1 dt/dx, c_1 = a1(x) dt/dv1, c_2 = a2 dt/dv2 and the
 // upwind neighbour f_u in each direction (zero beyond a velocity edge or the
@@ -282,16 +283,15 @@ step_direct_kernel(StepArgs a, int mode) {
   const Params& p = *a.prm;
   if (threadIdx.x == 0) s_flags = a.st->flags;
   __syncthreads();
-  // mode: kPassFull, kPassMoments (moments of f_in only), kPassX (x-advection
-  // with the wall and vacuum boundaries only), kPassV (v1, v2 advection,
-  // source and collisions only): these two make the Lie-split step;
+  // mode: kPassFull, kPassX (x-advection with the wall and vacuum boundaries
+  // only), kPassV (v1, v2 advection, source and collisions only): these two
+  // make the Lie-split step;
   // kPassXHalf and kPassXHalfLast (x-advection over dt/2, the second one
   // writing the partial sums of its output) with kPassV make the Strang step
-  const bool moments_only = mode == kPassMoments;
   const bool xlast = mode == kPassXHalfLast;
   const bool xpass = mode == kPassX || mode == kPassXHalf || xlast, vpass = mode == kPassV;
   const T xscale = (mode == kPassXHalf || xlast) ? (T)0.5 : (T)1;  // dt/2: exact halving
-  if (!moments_only && s_flags) return;  // sticky error: freeze the state
+  if (s_flags) return;  // sticky error: freeze the state
   const T* __restrict__ fin = static_cast<const T*>(a.f_in);
   T* __restrict__ fout = static_cast<T*>(a.f_out);
   const int nx = a.nx, nv1 = a.nv1, nv2 = a.nv2, pitch = a.pitch;
@@ -312,48 +312,45 @@ step_direct_kernel(StepArgs a, int mode) {
   const int ncell = (i1 - i0) * nv2;
   DensityAcc<T> s_n;
   double s_lv = 0.0, s_pe = 0.0, s_see = 0.0, s_vac = 0.0;
-  int neg = 0;  // a value written (or, moments only, read) is negative
+  int neg = 0;  // a value written is negative
   for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
     const int i = i0 + c / nv2;
     const int j = c - (c / nv2) * nv2;
     const size_t idx = (size_t)k * plane + (size_t)i * pitch + j;
     const size_t tix = (size_t)i * pitch + j;
     const T f = fin[idx];
-    T fn = f;
-    if (!moments_only) {
-      const T cx =
-          vpass ? (T)0 : xscale * (sizeof(T) == 8 ? (T)a.tab.cx[i] : (T)a.tab.cx32[i]);
-      T fx = (T)0;
-      if (cx > (T)0)
-        fx = k > 0 ? fin[idx - plane]
-                   : (T)(gsee * a.tab.gse[tix] +
-                         (p.refl > 0.0 ? p.refl * (double)fin[(size_t)(nv1 - 1 - i) * pitch + j]
-                                       : 0.0));
-      else if (cx < (T)0)
-        fx = k < nx - 1 ? fin[idx + plane] : (T)0;
-      T fv = (T)0;
-      if (c1 > (T)0)
-        fv = i > 0 ? fin[idx - pitch] : (T)0;
-      else if (c1 < (T)0)
-        fv = i < nv1 - 1 ? fin[idx + pitch] : (T)0;
-      T fw = (T)0;
-      if (c2 > (T)0)
-        fw = j > 0 ? fin[idx - 1] : (T)0;
-      else if (c2 < (T)0)
-        fw = j < nv2 - 1 ? fin[idx + 1] : (T)0;
-      T s = (T)0;
-      if (band) s = sizeof(T) == 8 ? (T)a.tab.src[tix] : (T)a.tab.src32[tix];
-      fn = update_cell<T>(f, fx, fv, fw, cx < (T)0 ? -cx : cx, a1, a2, s);
-      if (coll) {
-        const T m = sizeof(T) == 8 ? (T)(a.tab.m1[i] * a.tab.m2[j])
-                                   : (T)a.tab.m1_32[i] * (T)a.tab.m2_32[j];
-        fn += cs * m - ca * f;
-      }
-      fout[idx] = fn;
-      // loss through the downwind velocity edges, from f^n (ledger)
-      if ((c1 > (T)0 && i == nv1 - 1) || (c1 < (T)0 && i == 0)) s_lv += (double)a1 * (double)f;
-      if ((c2 > (T)0 && j == nv2 - 1) || (c2 < (T)0 && j == 0)) s_lv += (double)a2 * (double)f;
+    const T cx =
+        vpass ? (T)0 : xscale * (sizeof(T) == 8 ? (T)a.tab.cx[i] : (T)a.tab.cx32[i]);
+    T fx = (T)0;
+    if (cx > (T)0)
+      fx = k > 0 ? fin[idx - plane]
+                 : (T)(gsee * a.tab.gse[tix] +
+                       (p.refl > 0.0 ? p.refl * (double)fin[(size_t)(nv1 - 1 - i) * pitch + j]
+                                     : 0.0));
+    else if (cx < (T)0)
+      fx = k < nx - 1 ? fin[idx + plane] : (T)0;
+    T fv = (T)0;
+    if (c1 > (T)0)
+      fv = i > 0 ? fin[idx - pitch] : (T)0;
+    else if (c1 < (T)0)
+      fv = i < nv1 - 1 ? fin[idx + pitch] : (T)0;
+    T fw = (T)0;
+    if (c2 > (T)0)
+      fw = j > 0 ? fin[idx - 1] : (T)0;
+    else if (c2 < (T)0)
+      fw = j < nv2 - 1 ? fin[idx + 1] : (T)0;
+    T s = (T)0;
+    if (band) s = sizeof(T) == 8 ? (T)a.tab.src[tix] : (T)a.tab.src32[tix];
+    T fn = update_cell<T>(f, fx, fv, fw, cx < (T)0 ? -cx : cx, a1, a2, s);
+    if (coll) {
+      const T m = sizeof(T) == 8 ? (T)(a.tab.m1[i] * a.tab.m2[j])
+                                 : (T)a.tab.m1_32[i] * (T)a.tab.m2_32[j];
+      fn += cs * m - ca * f;
     }
+    fout[idx] = fn;
+    // loss through the downwind velocity edges, from f^n (ledger)
+    if ((c1 > (T)0 && i == nv1 - 1) || (c1 < (T)0 && i == 0)) s_lv += (double)a1 * (double)f;
+    if ((c2 > (T)0 && j == nv2 - 1) || (c2 < (T)0 && j == 0)) s_lv += (double)a2 * (double)f;
     s_n.add(fn);
     neg |= fn < (T)0;
     if (k == 0 && dir < 0) {
@@ -394,8 +391,111 @@ cudaError_t launch_step_pass(const StepArgs& a, int precision, int mode, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_step(const StepArgs& a, int precision, int moments_only, cudaStream_t s) {
-  return launch_step_pass(a, precision, moments_only ? kPassMoments : kPassFull, s);
+// ---------------------------------------------------------------------------
+// Moments of a state: the partial sums of f_in that a step writes of its
+// output, and the check for negative values.  One block per (plane, tile),
+// whose rows are one span of f (the row padding holds zeros), read 16 bytes a
+// load with eight loads in flight a thread; FP32 values go into a compensated
+// FP32 sum, FP64 ones into aligned 64-bit sums (fk_sum.cuh).  The wall and
+// vacuum sums take a second look at the two planes that have them.
+//
+// Bound by HBM at full size and by latency below.  With one cell a load and an
+// index division for each it took 116 us at 512 x 128 x 128 FP32; the five
+// evaluations of a grid set to a new point of a scan are 460 us shorter.
+constexpr int kMomThreads = 256;
+
+// a state has to hold no value below zero
+__device__ __forceinline__ bool below_zero(float x) { return x < 0.f; }
+__device__ __forceinline__ bool below_zero(double x) {
+  const int h = __double2hiint(x);
+  return h < 0 && ((h << 1) | __double2loint(x)) != 0;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_constant__ StepArgs a) {
+  __shared__ double sh[32];
+  constexpr int VEC = 16 / sizeof(T);
+  constexpr int L = kGroup * sizeof(double) / 16;  // loads in flight
+  const int nt = a.part.nu, nx = a.nx, pitch = a.pitch;
+  const int k = blockIdx.x / nt, t = blockIdx.x - k * nt;
+  int i0, i1, dir;
+  tile_rows(a.geom, a.nv1, t, &i0, &i1, &dir);
+  const T* span = static_cast<const T*>(a.f_in) + ((size_t)k * a.nv1 + i0) * pitch;
+  const int nvec = (i1 - i0) * pitch / VEC;
+  const float4* v = reinterpret_cast<const float4*>(span);
+  DensityAcc<T> acc;
+  int neg = 0;
+  for (int c0 = threadIdx.x; c0 - (int)threadIdx.x < nvec; c0 += kMomThreads * L) {
+    float4 w[L];
+#pragma unroll
+    for (int j = 0; j < L; j++) {
+      const int c = c0 + j * kMomThreads;
+      w[j] = c < nvec ? __ldg(v + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if constexpr (sizeof(T) == 8) {
+      double x[kGroup];
+#pragma unroll
+      for (int j = 0; j < L; j++) {
+        const double2 d = *reinterpret_cast<const double2*>(&w[j]);
+        x[2 * j] = d.x;
+        x[2 * j + 1] = d.y;
+      }
+#pragma unroll
+      for (int q = 0; q < kGroup; q++) neg |= below_zero(x[q]);
+      acc.s = add_group(x, acc.s);
+    } else {
+#pragma unroll
+      for (int j = 0; j < L; j++) {
+        const float x[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          neg |= below_zero(x[e]);
+          acc.add(x[e]);
+        }
+      }
+    }
+  }
+  if (__syncthreads_or(neg) && threadIdx.x == 0) atomicOr(&a.st->flags, kFlagNegative);
+  const double n_tot = block_sum<kMomThreads>(acc.value(), sh);
+  double pe = 0.0, see = 0.0, vac = 0.0;
+  const bool wall = k == 0 && dir < 0, vout = k == nx - 1 && dir > 0;
+  if (wall || vout) {
+    for (int c = threadIdx.x; c < (i1 - i0) * pitch; c += kMomThreads) {
+      const int i = i0 + c / pitch;
+      const double f = (double)span[c], v1 = a.tab.v1[i];
+      if (wall) {
+        pe = fma(-v1, f, pe);                                      // Eq. 13 without dv1 dv2
+        see = fma(a.tab.vdelta[(size_t)i0 * pitch + c], f, see);  // Eq. 12
+      } else {
+        vac = fma(v1, f, vac);
+      }
+    }
+    pe = block_sum<kMomThreads>(pe, sh);
+    see = block_sum<kMomThreads>(see, sh);
+    vac = block_sum<kMomThreads>(vac, sh);
+  }
+  if (threadIdx.x == 0) {
+    a.part.n[(size_t)k * nt + t] = n_tot;
+    a.part.lv[(size_t)k * nt + t] = 0.0;
+    if (k == 0) {
+      a.part.pe[t] = pe;
+      a.part.see[t] = see;
+    }
+    if (k == nx - 1) a.part.vac[t] = vac;
+  }
+}
+
+cudaError_t launch_moments(const StepArgs& a, int precision, cudaStream_t s) {
+  const int nblk = a.nx * a.part.nu;
+  if (precision == FK_F32)
+    moments_kernel<float><<<nblk, kMomThreads, 0, s>>>(a);
+  else
+    moments_kernel<double><<<nblk, kMomThreads, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_step(const StepArgs& a, int precision, cudaStream_t s) {
+  return launch_step_pass(a, precision, kPassFull, s);
 }
 
 __global__ void __launch_bounds__(kFinThreads)
