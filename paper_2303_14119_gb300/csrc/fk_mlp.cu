@@ -19,21 +19,21 @@ namespace fk {
 namespace {
 
 constexpr int kMTile = 128;   // rows per CTA (one MMA M)
-constexpr int kNTile = 64;    // columns per CTA (one MMA N at most)
+// columns per CTA (one MMA N at most): 64, or 32 where 64 leaves most SMs idle
+constexpr int kNTileWide = 64, kNTileThin = 32;
 constexpr int kNMax = 256;    // the largest N the entry points accept
 constexpr int kKChunk = 64;   // K per stage (4 MMAs of K = 16)
 constexpr int kGemmStages = 4;     // stages of the ring: K chunks in flight
-constexpr int kGemmThreads = 128;  // 4 warps: one per 32-lane slice of tensor memory
+constexpr int kGemmThreads = 256;  // 8 warps: two per 32-lane slice of tensor memory
 constexpr int kCoreBytes = 128;    // one 8 x 16-byte core matrix
 // a tile: [rows/8 row groups][kKChunk/8 K groups] core matrices
 constexpr int kLboBytes = kCoreBytes;                        // next core matrix along K
 constexpr int kSboBytes = (kKChunk / 8) * kCoreBytes;        // next 8-row group
 constexpr int kATileBytes = kMTile * kKChunk * 2;            // 16 KB
-constexpr int kBTileBytes = kNTile * kKChunk * 2;            // 8 KB
-constexpr int kGemmStageBytes = kATileBytes + kBTileBytes;   // 24 KB
+constexpr int gemm_stage_bytes(int nt) { return kATileBytes + nt * kKChunk * 2; }  // 20 or 24 KB
 // dynamic shared memory per CTA: the ring (two CTAs fit on an SM, with 2 x
 // 64 of its 512 tensor-memory columns)
-constexpr int kGemmSmem = kGemmStages * kGemmStageBytes;
+constexpr int gemm_smem(int nt) { return kGemmStages * gemm_stage_bytes(nt); }
 
 __device__ __forceinline__ uint16_t f32_to_bf16(float x) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(x));
@@ -80,6 +80,28 @@ __device__ __forceinline__ void stage_tile(unsigned char* dst, const uint16_t* s
   }
 }
 
+// Bias gradients: sums over the batch of the bf16 rows [r0, r0 + kMTile) of g.A,
+// each as 256 strided FP32 sums folded in trees of 32 and of 8, one warp a row.
+__device__ void row_sums_tile(const GemmArgs& g, int r0) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r = r0 + warp; r < min(r0 + kMTile, g.M); r += kGemmThreads / 32) {
+    const uint16_t* row = g.A + (long long)r * g.lda;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int c0 = 0; c0 < g.sum_n; c0 += 256)
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        const int c = c0 + 32 * j + lane;
+        if (c < g.sum_n) acc[j] += __uint_as_float((uint32_t)row[c] << 16);
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < 8; j++) acc[j] += __shfl_down_sync(0xffffffffu, acc[j], o);
+    if (lane == 0)
+      g.row_sum[r] = ((acc[0] + acc[4]) + (acc[2] + acc[6])) + ((acc[1] + acc[5]) + (acc[3] + acc[7]));
+  }
+}
+
 // One CTA: rows [m0, m0 + 128) x columns [n0, n0 + Nc) of C.  The K chunks
 // stream through a ring of kGemmStages shared-memory stages: every thread
 // queues its part of a chunk's copies (cp.async) up to kGemmStages chunks
@@ -87,14 +109,31 @@ __device__ __forceinline__ void stage_tile(unsigned char* dst, const uint16_t* s
 // commits them to the stage's mbarrier, whose phase frees the stage for
 // the chunk kGemmStages later.  Each output element sums its K terms in
 // the same order whatever the grid, so results are deterministic.
-template <int EPI>
-__global__ void __launch_bounds__(kGemmThreads) gemm_tn_kernel(const __grid_constant__ GemmArgs g) {
+//
+// At the network's sizes (256 x 256 x 256) the MMAs are a few percent: what
+// counts are the copies' latency and the epilogue, so eight warps share it,
+// with 16-byte stores; the GELU layers took 26 us with four warps of 64 columns
+// and one store an element.
+//
+// A launch holds up to three jobs (independent products, and the row sums of
+// an operand), one after the other in the grid.
+template <int kNTile>
+__global__ void __launch_bounds__(kGemmThreads) gemm_tn_kernel(const __grid_constant__ GemmJobs jobs) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint64_t bar[kGemmStages];
   __shared__ uint32_t s_taddr;
+  constexpr int kStageBytes = gemm_stage_bytes(kNTile);
+  int cta = blockIdx.x, job = 0;
+  while (cta >= jobs.ctas[job]) cta -= jobs.ctas[job++];
+  const GemmArgs& g = jobs.g[job];
+  const int mt = (g.M + kMTile - 1) / kMTile;
+  const int m0 = (cta % mt) * kMTile;
+  if (g.row_sum) {  // uniform over the CTA
+    row_sums_tile(g, m0);
+    return;
+  }
+  const int n0 = (cta / mt) * kNTile;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * kMTile;
-  const int n0 = blockIdx.y * kNTile;
   const int N = g.N;
   const int Nc = min(kNTile, (N + 15) / 16 * 16 - n0);  // this CTA's columns, a multiple of 16
   const uint32_t ncols = Nc <= 32 ? 32u : 64u;
@@ -113,7 +152,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tn_kernel(const __grid_cons
   const uint32_t idesc = tc::idesc_bf16_f32(kMTile, Nc);
   const int nch = (g.K + kKChunk - 1) / kKChunk;
   auto stage = [&](int c) {
-    unsigned char* sA = smem + (c % kGemmStages) * kGemmStageBytes;
+    unsigned char* sA = smem + (c % kGemmStages) * kStageBytes;
     stage_tile(sA, g.A, g.lda, m0, kMTile, g.M, c * kKChunk, g.K);
     stage_tile(sA + kATileBytes, g.B, g.ldb, n0, Nc, N, c * kKChunk, g.K);
     cp_async_commit();
@@ -130,7 +169,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tn_kernel(const __grid_cons
     __syncthreads();
     tc::fence_after_sync();
     if (tid == 0) {
-      const uint32_t a0 = tc::smem_u32(smem + q * kGemmStageBytes), b0 = a0 + kATileBytes;
+      const uint32_t a0 = tc::smem_u32(smem + q * kStageBytes), b0 = a0 + kATileBytes;
       for (int kk = 0; kk < kKChunk / 16; kk++) {
         // K step of 16 = two core matrices along K
         const uint64_t ad = tc::smem_desc(a0 + kk * 2 * kLboBytes, kLboBytes, kSboBytes);
@@ -151,34 +190,69 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tn_kernel(const __grid_cons
   }
   cp_async_wait(0);  // nothing left in flight into shared memory
   if (ok) {
-    // epilogue: warp w holds rows m0 + 32 w + lane (tensor-memory lanes)
-    const int row = m0 + warp * 32 + lane;
+    // epilogue: warps w and w + 4 hold rows m0 + 32 (w % 4) + lane (tensor-memory
+    // lanes), 16 columns of every 32 each
+    const int row = m0 + (warp & 3) * 32 + lane;
     const bool live = row < g.M;
-    for (int c0 = 0; c0 < Nc; c0 += 16) {
+    const bool whole = g.vec;  // 16-byte rows of C, H and Zin
+    for (int c0 = (warp >> 2) * 16; c0 < Nc; c0 += 32) {
       uint32_t r[16];
-      tc::tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
+      tc::tmem_ld16(taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, r);
       tc::tmem_wait_ld();
       if (!live) continue;
+      const int col0 = n0 + c0;
+      float v[16];
 #pragma unroll
       for (int e = 0; e < 16; e++) {
-        const int col = n0 + c0 + e;
-        if (col >= N) break;
-        float v = __uint_as_float(r[e]);
-        if (EPI == kEpiF32) {
-          if (g.bias) v += g.bias[col];
-          g.C[(long long)row * g.ldc + col] = v;
-        } else if (EPI == kEpiBiasGelu) {
-          const float z = v + (g.bias ? g.bias[col] : 0.f);
-          g.C[(long long)row * g.ldc + col] = z;
-          const uint16_t h = row < g.m_valid ? f32_to_bf16(gelu(z)) : (uint16_t)0;
-          g.H[(long long)row * g.ldh + col] = h;
-          if (g.Ht) g.Ht[(long long)col * g.ldht + row] = h;
-        } else {  // kEpiGeluBack
-          const float d = row < g.m_valid ? v * gelu_grad(g.Zin[(long long)row * g.ldz + col]) : 0.f;
-          const uint16_t h = f32_to_bf16(d);
-          g.H[(long long)row * g.ldh + col] = h;
-          if (g.Ht) g.Ht[(long long)col * g.ldht + row] = h;
+        v[e] = __uint_as_float(r[e]);
+        if (g.epi != kEpiGeluBack && g.bias && col0 + e < N) v[e] += g.bias[col0 + e];
+      }
+      const bool full = whole && col0 + 16 <= N;
+      if (g.epi != kEpiGeluBack) {
+        float* crow = g.C + (long long)row * g.ldc + col0;
+        if (full) {
+#pragma unroll
+          for (int e = 0; e < 16; e += 4)
+            *reinterpret_cast<float4*>(crow + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+        } else {
+          for (int e = 0; e < 16 && col0 + e < N; e++) crow[e] = v[e];
         }
+        if (g.epi == kEpiF32) continue;
+      }
+      float z[16];
+      if (g.epi == kEpiGeluBack) {
+        const float* zrow = g.Zin + (long long)row * g.ldz + col0;
+        if (full) {
+#pragma unroll
+          for (int e = 0; e < 16; e += 4)
+            *reinterpret_cast<float4*>(z + e) = *reinterpret_cast<const float4*>(zrow + e);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 16; e++) z[e] = col0 + e < N ? zrow[e] : 0.f;
+        }
+      }
+      uint32_t h[8];  // bf16 pairs
+#pragma unroll
+      for (int e = 0; e < 16; e++) {
+        float x = 0.f;
+        if (row < g.m_valid) x = g.epi == kEpiBiasGelu ? gelu(v[e]) : v[e] * gelu_grad(z[e]);
+        const uint32_t b = f32_to_bf16(x);
+        if (e & 1)
+          h[e / 2] |= b << 16;
+        else
+          h[e / 2] = b;
+      }
+      uint16_t* hrow = g.H + (long long)row * g.ldh + col0;
+      if (full) {
+        *reinterpret_cast<uint4*>(hrow) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(hrow + 8) = make_uint4(h[4], h[5], h[6], h[7]);
+      }
+#pragma unroll
+      for (int e = 0; e < 16; e++) {
+        if (col0 + e >= N) break;
+        const uint16_t x = (uint16_t)(h[e / 2] >> (16 * (e & 1)));
+        if (!full) hrow[e] = x;
+        if (g.Ht) g.Ht[(long long)(col0 + e) * g.ldht + row] = x;
       }
     }
   } else if (tid == 0) {
@@ -196,13 +270,24 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tn_kernel(const __grid_cons
   }
 }
 
-template <int EPI>
-cudaError_t launch_gemm_epi(const GemmArgs& g, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(gemm_tn_kernel<EPI>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+// CTAs of a job with kNTile-column tiles
+int job_ctas(const GemmArgs& g, int nt) {
+  const int mt = (g.M + kMTile - 1) / kMTile;
+  return g.row_sum ? mt : mt * (((g.N + 15) / 16 * 16 + nt - 1) / nt);
+}
+
+template <int kNTile>
+cudaError_t launch_jobs(GemmJobs& jobs, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(gemm_tn_kernel<kNTile>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(kNTile));
   if (e != cudaSuccess) return e;
-  const dim3 grid((g.M + kMTile - 1) / kMTile, ((g.N + 15) / 16 * 16 + kNTile - 1) / kNTile);
-  gemm_tn_kernel<EPI><<<grid, kGemmThreads, kGemmSmem, s>>>(g);
+  int total = 0;
+  for (int j = 0; j < kGemmJobs; j++) {
+    jobs.ctas[j] = j < jobs.n ? job_ctas(jobs.g[j], kNTile) : 0;
+    total += jobs.ctas[j];
+  }
+  jobs.ctas[jobs.n - 1] += 1 << 30;  // the search ends there
+  gemm_tn_kernel<kNTile><<<total, kGemmThreads, gemm_smem(kNTile), s>>>(jobs);
   return cudaGetLastError();
 }
 
@@ -225,26 +310,28 @@ __global__ void gather_kernel(const float* __restrict__ x_src, const float* __re
   }
 }
 
+// One warp per sample row: its share of dY in both layouts and its weighted
+// squared error.  (One thread summing a row's FP64 errors took 37 us.)
 __global__ void loss_grad_kernel(const float* __restrict__ Y, const float* __restrict__ T,
                                  const float* __restrict__ w, int n, int bp, int out_p,
                                  double inv_n, uint16_t* dY, uint16_t* dYt, double* loss_rows) {
-  const long long e = (long long)blockIdx.x * kEwThreads + threadIdx.x;
-  if (e < (long long)bp * out_p) {
-    const int r = (int)(e / out_p), c = (int)(e - (e / out_p) * out_p);
+  const int r = (int)((blockIdx.x * kEwThreads + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (r >= bp) return;
+  double acc = 0.0;
+  for (int c = lane; c < out_p; c += 32) {
+    const long long e = (long long)r * out_p + c;
     float d = 0.f;
-    if (r < n) d = (float)(2.0 * (double)w[c] * ((double)Y[e] - (double)T[e]) * inv_n);
+    if (r < n) {
+      const double dd = (double)Y[e] - (double)T[e], wc = (double)w[c];
+      d = (float)(2.0 * wc * dd * inv_n);
+      acc += wc * dd * dd;
+    }
     const uint16_t h = f32_to_bf16(d);
     dY[e] = h;
     dYt[(long long)c * bp + r] = h;
   }
-  if (e < n) {  // one thread per sample row: its weighted squared error
-    double acc = 0.0;
-    for (int c = 0; c < out_p; c++) {
-      const double dd = (double)Y[e * out_p + c] - (double)T[e * out_p + c];
-      acc += (double)w[c] * dd * dd;
-    }
-    loss_rows[e] = acc;
-  }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0 && r < n) loss_rows[r] = acc;
 }
 
 template <typename T>
@@ -261,15 +348,6 @@ __device__ __forceinline__ T block_reduce_sum(T v, T* sh) {
   return r;  // thread 0
 }
 
-__global__ void row_sums_kernel(const uint16_t* __restrict__ M, long long ld, int n, float* out) {
-  __shared__ float sh[32];
-  const uint16_t* row = M + (long long)blockIdx.x * ld;
-  float acc = 0.f;
-  for (int c = threadIdx.x; c < n; c += kEwThreads) acc += __uint_as_float((uint32_t)row[c] << 16);
-  acc = block_reduce_sum(acc, sh);
-  if (threadIdx.x == 0) out[blockIdx.x] = acc;
-}
-
 __global__ void loss_reduce_kernel(const double* __restrict__ rows, int n, double scale,
                                    double* acc) {
   __shared__ double sh[32];
@@ -279,17 +357,37 @@ __global__ void loss_reduce_kernel(const double* __restrict__ rows, int n, doubl
   if (threadIdx.x == 0) *acc += scale * v;
 }
 
-__global__ void adam_kernel(float* p, const float* __restrict__ g, float* m, float* v,
-                            long long count, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
+// Adam on every parameter, the bf16 copies of the new weights in both layouts,
+// and (the last block) the batch's loss: one launch instead of three and one
+// a layer.
+__global__ void __launch_bounds__(kEwThreads)
+adam_kernel(const __grid_constant__ AdamArgs a) {
+  __shared__ double sh[32];
+  if (blockIdx.x == gridDim.x - 1) {
+    double v = 0.0;
+    for (int r = threadIdx.x; r < a.n; r += kEwThreads) v += a.loss_rows[r];
+    v = block_reduce_sum(v, sh);
+    if (threadIdx.x == 0) *a.loss += a.loss_scale * v;
+    return;
+  }
   const long long e = (long long)blockIdx.x * kEwThreads + threadIdx.x;
-  if (e >= count) return;
-  const float gg = g[e];
-  const float mm = b1 * m[e] + (1.f - b1) * gg;
-  const float vv = b2 * v[e] + (1.f - b2) * gg * gg;
-  m[e] = mm;
-  v[e] = vv;
-  p[e] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+  if (e >= a.count) return;
+  const float gg = a.g[e];
+  const float mm = fmaf(1.f - a.b1, gg, a.b1 * a.m[e]);
+  const float vv = fmaf((1.f - a.b2) * gg, gg, a.b2 * a.v[e]);
+  a.m[e] = mm;
+  a.v[e] = vv;
+  const float p = a.p[e] - a.lr * (mm / a.c1) / (sqrtf(vv / a.c2) + a.eps);
+  a.p[e] = p;
+  int q = 0;
+  while (q + 1 < a.layers && e >= a.woff[q + 1]) q++;
+  const long long w = e - a.woff[q];
+  const int K = a.K[q], N = a.N[q];
+  if (w >= (long long)N * K) return;  // a bias
+  const int r = (int)(w / K), c = (int)(w - (w / K) * K);
+  const uint16_t h = f32_to_bf16(p);
+  a.Wb[q][w] = h;
+  a.Wt[q][(long long)c * N + r] = h;
 }
 
 __global__ void pack_weights_kernel(const float* __restrict__ W, int N, int K, uint16_t* Wb,
@@ -318,14 +416,8 @@ cudaError_t launch_gather(const float* x_src, const float* t_src, const int* idx
 cudaError_t launch_loss_grad(const float* Y, const float* T, const float* w, int n, int bp,
                              int out_p, double inv_n, uint16_t* dY, uint16_t* dYt,
                              double* loss_rows, cudaStream_t s) {
-  loss_grad_kernel<<<ew_blocks((long long)bp * out_p), kEwThreads, 0, s>>>(
+  loss_grad_kernel<<<ew_blocks((long long)bp * 32), kEwThreads, 0, s>>>(
       Y, T, w, n, bp, out_p, inv_n, dY, dYt, loss_rows);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_row_sums(const uint16_t* M, long long ld, int rows, int n, float* out,
-                            cudaStream_t s) {
-  row_sums_kernel<<<rows, kEwThreads, 0, s>>>(M, ld, n, out);
   return cudaGetLastError();
 }
 
@@ -335,13 +427,12 @@ cudaError_t launch_loss_reduce(const double* loss_rows, int n, double scale, dou
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(float* p, const float* g, float* m, float* v, long long count, float lr,
-                        float b1, float b2, float eps, int t, cudaStream_t s) {
+cudaError_t launch_adam(AdamArgs a, int t, cudaStream_t s) {
   // bias corrections 1 - beta^t in FP64: in FP32, 1 - 0.999^t loses about
   // nine bits to cancellation at small t
-  const float c1 = (float)(1.0 - pow((double)b1, (double)t));
-  const float c2 = (float)(1.0 - pow((double)b2, (double)t));
-  adam_kernel<<<ew_blocks(count), kEwThreads, 0, s>>>(p, g, m, v, count, lr, b1, b2, eps, c1, c2);
+  a.c1 = (float)(1.0 - pow((double)a.b1, (double)t));
+  a.c2 = (float)(1.0 - pow((double)a.b2, (double)t));
+  adam_kernel<<<ew_blocks(a.count) + 1, kEwThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -362,10 +453,25 @@ const char* gemm_shape_error(const GemmArgs& g) {
   return nullptr;
 }
 
-cudaError_t launch_gemm(const GemmArgs& g, int epi, cudaStream_t s) {
-  if (epi == kEpiF32) return launch_gemm_epi<kEpiF32>(g, s);
-  if (epi == kEpiBiasGelu) return launch_gemm_epi<kEpiBiasGelu>(g, s);
-  return launch_gemm_epi<kEpiGeluBack>(g, s);
+cudaError_t launch_gemms(const GemmArgs* g, int n, cudaStream_t s) {
+  GemmJobs jobs{};
+  jobs.n = n;
+  int wide = 0;
+  for (int j = 0; j < n; j++) {
+    jobs.g[j] = g[j];
+    GemmArgs& x = jobs.g[j];
+    const uintptr_t ptrs = (uintptr_t)x.C | (uintptr_t)x.H | (uintptr_t)x.Zin;
+    x.vec = !(ptrs & 15) && !(x.ldc % 4) && !(x.ldh % 8) && !(x.ldz % 4);
+    if (!x.row_sum) wide += job_ctas(x, kNTileWide);
+  }
+  // half-width tiles while even those leave the GPU half empty (512 x 256 x 256: 16 CTAs
+  // of 64 columns, 32 of 32)
+  return wide <= 76 ? launch_jobs<kNTileThin>(jobs, s) : launch_jobs<kNTileWide>(jobs, s);
+}
+
+cudaError_t launch_gemm(GemmArgs g, int epi, cudaStream_t s) {
+  g.epi = epi;
+  return launch_gemms(&g, 1, s);
 }
 
 }  // namespace fk

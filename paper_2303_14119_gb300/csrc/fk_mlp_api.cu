@@ -146,6 +146,27 @@ GemmArgs gemm_args(fk_mlp* m) {
   return g;
 }
 
+AdamArgs adam_args(fk_mlp* m) {
+  AdamArgs a{};
+  a.p = m->d_p;
+  a.m = m->d_m;
+  a.v = m->d_v;
+  a.g = m->d_g;
+  a.count = (long long)m->np;
+  a.b1 = 0.9f;
+  a.b2 = 0.999f;
+  a.eps = 1e-8f;
+  a.layers = m->L;
+  for (int q = 0; q < m->L; q++) {
+    a.K[q] = m->K[q];
+    a.N[q] = m->N[q];
+    a.woff[q] = (long long)m->woff[q];
+    a.Wb[q] = m->Wb[q];
+    a.Wt[q] = m->Wt[q];
+  }
+  return a;
+}
+
 // Forward pass over bp rows (n live) from H[0] / Ht[0]: hidden layers with
 // the bias + GELU epilogue (Z kept for the backward pass), output layer with
 // the bias epilogue into Y.
@@ -188,6 +209,8 @@ fk_status backward_pass(fk_mlp* m, int n, int bp, double inv_n) {
   const uint16_t* dzt = m->d_dYt;  // [N_q][bp]
   int cur = 0;
   for (int q = m->L - 1; q >= 0; q--) {
+    // all three read this layer's dZ: one launch
+    GemmArgs jobs[3];
     GemmArgs g = gemm_args(m);
     g.A = dzt;
     g.lda = bp;
@@ -199,9 +222,19 @@ fk_status backward_pass(fk_mlp* m, int n, int bp, double inv_n) {
     g.C = m->d_g + m->woff[q];
     g.ldc = m->K[q];
     g.m_valid = m->N[q];
-    MK_CUDA(m, launch_gemm(g, kEpiF32, m->stream));
-    MK_CUDA(m, launch_row_sums(dzt, bp, m->N[q], n, m->d_g + m->boff[q], m->stream));
-    if (q == 0) break;
+    g.epi = kEpiF32;
+    GemmArgs bsum = gemm_args(m);
+    bsum.A = dzt;
+    bsum.lda = bp;
+    bsum.M = m->N[q];
+    bsum.row_sum = m->d_g + m->boff[q];
+    bsum.sum_n = n;
+    if (q == 0) {
+      jobs[0] = g;
+      jobs[1] = bsum;
+      MK_CUDA(m, launch_gemms(jobs, 2, m->stream));
+      break;
+    }
     GemmArgs d = gemm_args(m);
     d.A = dz;
     d.lda = m->N[q];
@@ -217,7 +250,11 @@ fk_status backward_pass(fk_mlp* m, int n, int bp, double inv_n) {
     d.Ht = m->d_dZt[cur];
     d.ldht = bp;
     d.m_valid = n;
-    MK_CUDA(m, launch_gemm(d, kEpiGeluBack, m->stream));
+    d.epi = kEpiGeluBack;
+    jobs[0] = d;  // on the way of the next layer
+    jobs[1] = g;
+    jobs[2] = bsum;
+    MK_CUDA(m, launch_gemms(jobs, 3, m->stream));
     dz = m->d_dZ[cur];
     dzt = m->d_dZt[cur];
     cur ^= 1;
@@ -519,15 +556,14 @@ fk_status fk_mlp_train(fk_mlp* m, const float* x, const float* t, const float* w
         release();
         return s;
       }
-      TRAIN_CUDA(launch_loss_reduce(m->d_lrow, nb, 1.0 / (double)n, dl + ep, m->stream));
       m->adam_t += 1;
-      TRAIN_CUDA(launch_adam(m->d_p, m->d_g, m->d_m, m->d_v, (long long)m->np, lr, 0.9f, 0.999f,
-                             1e-8f, (int)std::min<long long>(m->adam_t, 1 << 30), m->stream));
-      s = pack_all(m);
-      if (s != FK_OK) {
-        release();
-        return s;
-      }
+      AdamArgs ad = adam_args(m);
+      ad.lr = lr;
+      ad.loss_rows = m->d_lrow;
+      ad.n = nb;
+      ad.loss_scale = 1.0 / (double)n;
+      ad.loss = dl + ep;
+      TRAIN_CUDA(launch_adam(ad, (int)std::min<long long>(m->adam_t, 1 << 30), m->stream));
     }
     // the host permutation is rewritten next epoch: its copy must be done
     TRAIN_CUDA(cudaStreamSynchronize(m->stream));
