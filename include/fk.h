@@ -31,7 +31,7 @@
  *    the status.  Where f is checked for negative values: every cell of a
  *    state set with fk_set_f / fk_set_f32 (the call returns FK_ENEGATIVE),
  *    every cell a direct-load pass writes, and the wall and vacuum planes of
- *    every streaming step or split-scheme pass on the streaming kernel.  The
+ *    every streaming step, split step or pass of one.  The
  *    interior of a streaming pass is not checked per cell: with f >= 0 and
  *    the Courant sum (checked every step) at most 1, its update is a sum of
  *    non-negative terms.
@@ -198,10 +198,11 @@ fk_status fk_set_reflection(fk_grid *grid, double R_f);
  * x-advection over dt/2; each x half-step takes its wall fluxes (Eqs. 12-15)
  * from its own input state, so the surface charge and the wall ledger terms
  * take dt/2 of the fluxes of f^n and dt/2 of those of the state after the
- * velocity step.  Sec. 2 states only an explicit upwind update; the split
- * forms run as two (Lie) or three (Strang) passes over f through one more
- * buffer of f: each pass is the streaming step kernel with the other terms'
- * coefficients zeroed (the direct-load kernel on grids too wide for it),
+ * velocity step.  Sec. 2 states only an explicit upwind update.  A split step
+ * is one pass over f (a kernel of its own); on grids too wide for its tiles it
+ * runs as two (Lie) or three (Strang) passes through one more buffer of f,
+ * each the streaming step kernel with the other terms' coefficients zeroed
+ * (the direct-load kernel on grids too wide for that),
  * and grids using them cannot join a batch.  FK_EINVAL for another value;
  * FK_ESTATE while the grid is in a batch. */
 #define FK_SCHEME_UNSPLIT 0

@@ -16,6 +16,7 @@
 
 #include "fk_host.cuh"
 #include "fk_resident.cuh"
+#include "fk_split.cuh"
 
 using namespace fk;
 
@@ -229,13 +230,33 @@ fk_status evaluate(fk_grid* g, int mode) {
   return FK_OK;
 }
 
+// The fused split step's arguments: its own tiles and partial sums.
+SplitArgs split_args(fk_grid* g, const StepArgs& step) {
+  SplitArgs sa{};
+  sa.a = step;
+  sa.a.geom = g->split_geom[g->scheme == kSchemeStrang];
+  const int nt = sa.a.geom.n_tiles;
+  const size_t np = (size_t)g->nx * nt;
+  double* b = g->d_split_part;
+  sa.a.part = Partials{b, b + np, b + 2 * np, b + 2 * np + nt, b + 2 * np + 2 * nt, nt};
+  sa.pe_mid = b + 2 * np + 3 * nt;
+  sa.see_mid = sa.pe_mid + nt;
+  sa.vac_mid = sa.see_mid + nt;
+  sa.h_wall = g->d_h_wall;
+  return sa;
+}
+
 // One step: the step kernel then the finalize kernel on stream s.
 cudaError_t enqueue_step(fk_grid* g, int cur, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1) {
   StepArgs a = make_args(g, cur);
   cudaError_t e = cudaSuccess;
   if (ev0) e = cudaEventRecord(ev0, s);
   if (e == cudaSuccess) {
-    if (g->scheme != kSchemeUnsplit && g->use_stream) {
+    if (g->scheme != kSchemeUnsplit && g->split_geom[0].n_tiles > 0) {
+      const SplitArgs sa = split_args(g, a);
+      e = launch_split_step(sa, g->prec, g->scheme == kSchemeStrang, g->prm.collisions != 0, s);
+      a.part = sa.a.part;  // what the finalize folds
+    } else if (g->scheme != kSchemeUnsplit && g->use_stream) {
       // the split steps' passes on the streaming kernel: an x pass is the
       // fused step with c_1 = c_2 = 0, no source and no collisions (c_x / 2
       // for a Strang half pass); the velocity pass is the fused step with
@@ -377,7 +398,7 @@ void free_grid(fk_grid* g) {
                   g->d_bgk, g->d_bgk32, g->part.n, g->part.lv,
                   g->part.pe, g->part.see, g->d_res, g->d_lv_odd,
                   g->part.vac, g->d_ne, g->d_Ex, g->d_c1, g->d_c1_32, g->d_hist,
-                  g->d_stage, g->d_f3, g->d_st_mid, g->d_prm_x, g->d_zero, g->d_cx_half,
+                  g->d_stage, g->d_split_part, g->d_h_wall, g->d_f3, g->d_st_mid, g->d_prm_x, g->d_zero, g->d_cx_half,
                   g->d_cx32_half, g->d_lv_aside, g->fin.pre, g->fin.bsum, g->fin.blv,
                   g->fin.counter};
   for (void* p : ptrs)
@@ -394,9 +415,23 @@ cudaError_t dalloc(P** p, size_t bytes) {
   return hooked_alloc(reinterpret_cast<void**>(p), bytes ? bytes : 16);
 }
 
-// The buffers a time scheme needs beyond the two state buffers: a third
-// buffer of f for the split steps, and the Strang step's second state block.
+// The buffers a time scheme needs beyond the two state buffers.  Fused split
+// steps: their partial sums and boundary planes.  Split steps as passes: a
+// third buffer of f, and the Strang step's second state block.
 fk_status split_buffers(fk_grid* g, int scheme) {
+  if (scheme != kSchemeUnsplit && g->split_geom[0].n_tiles > 0) {
+    const size_t n = (2 * (size_t)g->nx + 6) * g->split_geom[0].n_tiles * sizeof(double);
+    if (!g->d_split_part) {
+      FK_CUDA(g, dalloc(&g->d_split_part, n));
+      FK_CUDA(g, cudaMemsetAsync(g->d_split_part, 0, n, g->stream));
+    }
+    if (!g->d_h_wall) {
+      const size_t hb = (size_t)g->nv1 * g->pitch * g->esize;
+      FK_CUDA(g, dalloc(&g->d_h_wall, hb));
+      FK_CUDA(g, cudaMemsetAsync(g->d_h_wall, 0, hb, g->stream));
+    }
+    return FK_OK;
+  }
   if (scheme != kSchemeUnsplit && !g->d_f3)
     FK_CUDA(g, dalloc(&g->d_f3, (size_t)g->nx * g->nv1 * g->pitch * g->esize));
   if (scheme == kSchemeStrang && !g->d_st_mid) {
@@ -528,6 +563,12 @@ fk_status plan_geometry(fk_grid* g) {
     }
   }
   plan_resident(g, sms);
+  Geom sg[2]{};
+  if (g->use_stream && plan_split(g->prec, false, g->nx, g->nv1, g->pitch, i_neg, sms, &sg[0]) &&
+      plan_split(g->prec, true, g->nx, g->nv1, g->pitch, i_neg, sms, &sg[1])) {
+    g->split_geom[0] = sg[0];
+    g->split_geom[1] = sg[1];
+  }
   return FK_OK;
 }
 

@@ -61,9 +61,17 @@ struct fk_grid {
   int ev_used = 0;              // pairs recorded since the last read
   // batch that steps this grid: while set, calls that change the state are
   // refused and the getters wait for the batch's last enqueued step
-  int scheme = 0;             // kSchemeUnsplit or kSchemeLie
-  void* d_f3 = nullptr;       // intermediate state of the split steps
-  // the split steps' passes on the streaming kernel: the parameters of an
+  int scheme = 0;             // kSchemeUnsplit, kSchemeLie or kSchemeStrang
+  // the fused split steps (fk_split.cu): the tiles of a Lie and of a Strang
+  // step (none: the steps run as passes; the two differ in their chunks
+  // only), their partial sums in one buffer and the boundary planes of the
+  // state after the velocity step
+  fk::Geom split_geom[2]{};
+  double* d_split_part = nullptr;
+  void* d_h_wall = nullptr;
+  // the split steps as passes: an intermediate state of f
+  void* d_f3 = nullptr;
+  // the passes on the streaming kernel: the parameters of an
   // x pass (c_2 = 0, no source band, no collisions), zeros for the c_1 of
   // an x pass and the c_x of the velocity pass (one array of
   // max(nx, nv1) doubles, which read as floats are zeros too), c_x / 2 of
