@@ -25,7 +25,7 @@
 // that holds the wall; on large ones HBM.  Measured, us a step, two launches
 // a step replayed as graphs -> here: 64 x 48 x 48 FP64 34.7 -> 16.1, FP32 21.8
 // -> 9.8; 321 x 117 x 117 FP32 25.9 -> 21.6; 512 x 128 x 128 FP32 with
-// collisions 32.9 -> 24.1; 1024 x 256 x 256 FP32 109.8 -> 101.4, FP64 622 -> 607.
+// collisions 32.9 -> 24.1; 1024 x 256 x 256 FP32 109.8 -> 101.4, FP64 622 -> 574.
 //
 // Waits: every block of the launch is resident (cooperative launch), every
 // wait is bounded by Params::wait_limit, and after one that runs out the

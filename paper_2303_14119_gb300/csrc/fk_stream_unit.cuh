@@ -199,7 +199,8 @@ __host__ __device__ constexpr size_t stage_bytes(int stage_elems) {
 // a grid stepped alone or in a batch.  After the slot and the stages come:
 // mbarriers full[NS], empty[NS] (NS stages); warp sums [NS][kWarps][4]
 // (a half unit uses the first 3 warps of each stage)
-// (density, wall primary flux, wall secondary flux, vacuum outflow); for
+// (density as one or two floats, wall primary flux, wall secondary flux,
+// vacuum outflow); for
 // FP64 grids the per-stage diagonal 1 - |c_x| - |c_1| - |c_2| (- dt nu) of
 // every tile row [NS][kMaxTileRows] double, for FP32 grids the
 // separable source factors of the tile rows [kMaxTileRows] and of the row
@@ -857,14 +858,14 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
     struct Gathered {
       int k;       // plane (-1: the prime item, no sums)
       T lvt;       // this lane's share of the velocity-edge outflow
-      float wsf;   // lane w < NW, FP32 grids: warp w's density sum
-      double ws[kWs];  // lane w < NW: warp w's sums (all four on a wall plane)
+      float2 wsf;  // lane w < NW: warp w's density sum (FP64 grids: hi, lo)
+      double ws[kWs];  // lane w < NW: warp w's other sums, on a wall plane
     };
     auto gather = [&](int q) -> Gathered {
       Gathered g;
       g.k = -1;
       g.lvt = (T)0;
-      g.wsf = 0.f;
+      g.wsf = make_float2(0.f, 0.f);
 #pragma unroll
       for (int i = 0; i < kWs; i++) g.ws[i] = 0.0;
       if (prime && q == 0) return g;
@@ -889,9 +890,10 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
         for (int r = lane; r < rows; r += 32) g.lvt += a2t * sb[(size_t)(r + rb) * pitch + nv2 - 1];
       if (lane < NW) {
         const double* ws = wsum + (st * kWarps + lane) * kWs;
-        // FP32 grids hand over their warp's density sum as a float
-        g.ws[0] = sizeof(T) == 4 ? (double)0 : ws[0];
-        if constexpr (sizeof(T) == 4) g.wsf = *reinterpret_cast<const float*>(ws);
+        if constexpr (sizeof(T) == 4)
+          g.wsf.x = *reinterpret_cast<const float*>(ws);
+        else
+          g.wsf = *reinterpret_cast<const float2*>(ws);
         if (k == 0 || k == nx - 1) {
 #pragma unroll
           for (int i = 1; i < kWs; i++) g.ws[i] = ws[i];
@@ -907,19 +909,29 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
       const double lv = (double)warp_sum(g.lvt);
       double sum[kWs] = {0.0, 0.0, 0.0, 0.0};
       const bool wall = k == 0 || k == nx - 1;
-      float sumf = 0.f;  // FP32 grids: the warps' density sums, added in FP32
+      if constexpr (sizeof(T) == 4) {  // added in FP32, one conversion per plane
+        float sumf = 0.f;
 #pragma unroll
-      for (int w = 0; w < NW; w++) {
-        if constexpr (sizeof(T) == 4)
-          sumf += __shfl_sync(0xffffffffu, g.wsf, w);
-        else
-          sum[0] += __shfl_sync(0xffffffffu, g.ws[0], w);
-        if (wall) {
+        for (int w = 0; w < NW; w++) sumf += __shfl_sync(0xffffffffu, g.wsf.x, w);
+        sum[0] = (double)sumf;
+      } else {
+        // An FP64 instruction takes the SM's FP64 pipe 16 cycles, for one lane
+        // as for 32, and that pipe bounds FP64 grids: the warps' pairs become
+        // FP64 here, all at once, and are folded in a tree.  With the
+        // conversions in each consumer warp and a serial fold a plane of 13 rows
+        // of 256 took 40 FP64 instructions beside its 416 for the update: 603 us
+        // a step at 1024 x 256 x 256, now 574; 512 x 128 x 128 92 -> 88 us.
+        sum[0] = (double)g.wsf.x + (double)g.wsf.y;
+#pragma unroll
+        for (int o = NW > 4 ? 4 : 2; o > 0; o >>= 1)
+          sum[0] += __shfl_down_sync(0xffffffffu, sum[0], o);
+      }
+      if (wall) {
+#pragma unroll
+        for (int w = 0; w < NW; w++)
 #pragma unroll
           for (int i = 1; i < kWs; i++) sum[i] += __shfl_sync(0xffffffffu, g.ws[i], w);
-        }
       }
-      if constexpr (sizeof(T) == 4) sum[0] = (double)sumf;  // one conversion per plane
       if (lane == 0 && in_bounds(k >= 0 && k < nx && t >= 0 && t < nt, a.st)) {
         a.part.n[(size_t)k * nt + t] = sum[0];
         lvp[(size_t)k * nt + t] = lv;
@@ -1307,7 +1319,8 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
           const T ws = warp_sum(sum_n);
           if (lane == 0) *reinterpret_cast<float*>(wsl) = ws;  // the producer converts once
         } else {
-          // fold the lanes' (hi, error) pairs in FP32 with TwoSum, convert once
+          // fold the lanes' (hi, error) pairs in FP32 with TwoSum; the producer
+          // converts them
           float lo = sc_ + sl_;
           for (int o = 16; o > 0; o >>= 1) {
             const float oh = __shfl_down_sync(0xffffffffu, sh_, o);
@@ -1316,7 +1329,7 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
             two_sum_acc(sh_, c, oh);
             lo += ol + c;
           }
-          if (lane == 0) wsl[0] = (double)sh_ + (double)lo;
+          if (lane == 0) *reinterpret_cast<float2*>(wsl) = make_float2(sh_, lo);
         }
         const bool wall = !RES && k == 0 && dir < 0, vout = !RES && k == nx - 1 && dir > 0;
         if (wall || vout) {  // uniform over the block
