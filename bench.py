@@ -180,7 +180,7 @@ class ClockSampler:
 
 # --------------------------------------------------------------- our arm
 SCHEMES = {"unsplit": 0, "lie": 1, "strang": 2}
-PASSES = {"unsplit": 1, "lie": 2, "strang": 3}  # passes over f per step
+FP64_OPS = {"unsplit": 4, "lie": 5, "strang": 7}  # FP64 operations a cell and step
 
 
 def make_grids(fk, w, precision, stream, phys=None):
@@ -303,10 +303,11 @@ def time_arm(fk, torch, w, precision, f0, steps, warmup, dist, device, batch=Tru
         plan = dict(mode="per-instance", timed="CUDA-graph replay per instance",
                     **{k: info[k] for k in ("kernel", "n_tiles", "n_chunks", "chunk_len")})
         cells_per_launch = cells
-        # per step: the pass(es), the Strang mid-step fold, the finalize
+        # split steps: the march, the Strang step's x = 0 plane, the finalize;
+        # unsplit steps of one grid: up to 128 in a launch
         scheme = phys["scheme"] if phys else "unsplit"
-        per_step = {"unsplit": 2, "lie": 3, "strang": 5}[scheme]
-        gpu_launches = per_step * steps * len(grids)
+        per_grid = {"unsplit": -(-steps // 128), "lie": 2 * steps, "strang": 3 * steps}[scheme]
+        gpu_launches = per_grid * len(grids)
     return dict(ms=ms, launches=launches, kernel_ms=kms, cells=cells, n_inst=len(grids),
                 cells_per_launch=cells_per_launch, gpu_launches=gpu_launches, clocks=ck,
                 grids=grids, kernel=plan)
@@ -433,18 +434,17 @@ def cpu_baseline(w, seconds=10.0):
 # FMA per cycle x 2.07 GHz = 0.629 T FMA/s = 1.26 TFLOP/s (NVIDIA's figure is
 # 1.25 TFLOP/s; a register-resident FMA loop measured 0.596 T FMA/s).
 FP64_PEAK_TFLOPS = 152 * 2 * 2.07e9 * 2 / 1e12
-DFMA_PER_CELL = 4  # the FP64 update is four fused multiply-adds per cell
 
 
-def roofline(res, precision, peak, peak_kind, workload, passes=1, plain=True):
-    """passes: passes over f per timed launch (one read of f and one write
-    each; the split schemes' passes are timed together); plain: the
+def roofline(res, precision, peak, peak_kind, workload, scheme="unsplit", plain=True):
+    """One read and one write of f per timed launch, whatever the scheme (a
+    Strang step's small second kernel is timed with it); plain: the
     workload's default physics, the only case the traffic record covers."""
     bpc = 4 if precision == "f32" else 8
     if res["launches"] == 0:
         return None
     avg_s = res["kernel_ms"] / res["launches"] / 1e3
-    alg_bytes = passes * 2 * bpc * res["cells_per_launch"]  # one read of f^n, one write of f^{n+1}
+    alg_bytes = 2 * bpc * res["cells_per_launch"]  # one read of f^n, one write of f^{n+1}
     achieved = alg_bytes / avg_s / 1e9
     hbm = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
            "frac": round(achieved / peak, 4),
@@ -454,9 +454,8 @@ def roofline(res, precision, peak, peak_kind, workload, passes=1, plain=True):
            "alg_bytes_per_launch": alg_bytes}
     if precision == "f32":
         return hbm
-    # FP64 on GB300 is bound by the FP64 pipe, not by HBM (every pass of a
-    # split step runs the fused update, four DFMA per cell)
-    flops = passes * 2 * DFMA_PER_CELL * res["cells_per_launch"]
+    # FP64 on GB300 is bound by the FP64 pipe, not by HBM
+    flops = 2 * FP64_OPS[scheme] * res["cells_per_launch"]
     tflops = flops / avg_s / 1e12
     return {"bound": "alu", "achieved": round(tflops, 4), "peak": round(FP64_PEAK_TFLOPS, 4),
             "unit": "TFLOP/s", "frac": round(tflops / FP64_PEAK_TFLOPS, 4),
@@ -488,7 +487,6 @@ def run_ours(args):
     plain = not args.collisions and args.reflection == 0.0 and args.scheme == "unsplit"
     # batches step the unsplit scheme only: a split scheme steps each instance alone
     batch = not args.no_batch and args.scheme == "unsplit"
-    passes = PASSES[args.scheme]
     res = time_arm(fk, torch, w, prec, f0, args.steps, args.warmup, dist, local,
                    batch=batch, chunk_len=args.chunk_len, tile_rows=args.tile_rows, phys=phys)
     for g in res.pop("grids"):
@@ -504,7 +502,7 @@ def run_ours(args):
                    "cells_per_instance": res["cells"], "precision_storage": args.precision,
                    "accumulators": "f64", "l2": "inputs larger than L2 (no flush)",
                    "parallelism": "replicas" if world > 1 else "single GPU"},
-        "roofline": roofline(res, args.precision, peak, peak_kind, args.workload, passes, plain),
+        "roofline": roofline(res, args.precision, peak, peak_kind, args.workload, args.scheme, plain),
         "kernel_plan": res["kernel"],
         "gpu_launches": res["gpu_launches"],
         "clocks": res["clocks"],
@@ -513,8 +511,7 @@ def run_ours(args):
         line["config"]["physics"] = dict(
             collisions="BGK, T_e 2 eV, ln Lambda 10" if args.collisions else "off",
             reflection=args.reflection, scheme=args.scheme,
-            passes_per_step=passes, timed_launches=("the step kernel" if passes == 1 else
-                                                    "the %d passes of a step together" % passes))
+            passes_per_step=1, timed_launches="the step kernel")
     if not args.no_side:
         other = "f64" if args.precision == "f32" else "f32"
         oprec = fk.FK_F64 if other == "f64" else fk.FK_F32
@@ -526,7 +523,7 @@ def run_ours(args):
         line["side_by_side"] = {other: {
             "value": world * r2["n_inst"] * r2["cells"] * osteps / (r2["ms"] / 1e3),
             "ms_per_step": r2["ms"] / osteps, "steps": osteps,
-            "roofline": roofline(r2, other, peak, peak_kind, args.workload, passes, plain),
+            "roofline": roofline(r2, other, peak, peak_kind, args.workload, args.scheme, plain),
             "clocks": r2["clocks"]}}
     if not args.no_e2e:
         e2e_steps = args.e2e_steps or min(int(w.get("steps", 100)), 20000)

@@ -15,7 +15,7 @@
 //
 // Measured, us a step, passes -> here: Strang 512 x 128 x 128 FP32 66 -> 44,
 // FP64 270 -> 164, 1024 x 256 x 256 FP32 309 -> 162, 64 x 48 x 48 FP64 85 ->
-// 36; Lie 1024 x 256 x 256 FP32 207 -> 118, 512 x 256 x 256 FP64 623 -> 427.
+// 37; Lie 1024 x 256 x 256 FP32 207 -> 118, 512 x 256 x 256 FP64 623 -> 429.
 // Small grids are bound by the launches and the finalize, FP64 grids by the
 // FP64 pipe (5 operations a cell for Lie and 7 for Strang, where the passes
 // took 8 and 12), large FP32 ones by the latency of a plane's two phases.
@@ -69,21 +69,23 @@ __host__ __device__ constexpr size_t split_smem_bytes(int stage_elems, int pitch
   return kSplitStages * stage_bytes<T>(stage_elems) + split_tail_bytes<T>(pitch);
 }
 
-// x-step of one cell.  Increment form: exact where nothing flows, and >= 0
-// for f, fx >= 0 and ax <= 1 (fx - f rounds to -f or more).
-__device__ __forceinline__ double x_step(double f, double fx, double ax) { return fma(ax, fx - f, f); }
-__device__ __forceinline__ float x_step(float f, float fx, float ax) { return fmaf(ax, fx - f, f); }
-
-__device__ __forceinline__ Vec<double> x_step_vec(const Vec<double>& f, const double (&fx)[2], double ax) {
-  Vec<double> r;
-  r.e[0] = x_step(f.e[0], fx[0], ax);
-  r.e[1] = x_step(f.e[1], fx[1], ax);
-  return r;
+// x-step of one cell, in the streaming kernel's arithmetic: convex form of
+// FP64 grids (d = 1 - ax), increment form of FP32 grids.
+__device__ __forceinline__ double x_step(double f, double fx, double ax, double d) {
+  return fma(ax, fx, d * f);
 }
-__device__ __forceinline__ Vec<float> x_step_vec(const Vec<float>& f, const float (&fx)[4], float ax) {
+__device__ __forceinline__ float x_step(float f, float fx, float ax, float) {
+  return __fadd_rn(f, __fmul_rn(ax, fx - f));
+}
+__device__ __forceinline__ Vec<double> x_step_vec(const Vec<double>& f, const double (&fx)[2], double ax,
+                                                  double d) {
+  return Vec<double>{{x_step(f.e[0], fx[0], ax, d), x_step(f.e[1], fx[1], ax, d)}};
+}
+__device__ __forceinline__ Vec<float> x_step_vec(const Vec<float>& f, const float (&fx)[4], float ax,
+                                                 float) {
   const F2 f0 = f2_pack(f.e[0], f.e[1]), f1 = f2_pack(f.e[2], f.e[3]), a2 = f2_pack(ax, ax);
-  const float2 r0 = f2_unpack(f2_fma(a2, f2_sub(f2_pack(fx[0], fx[1]), f0), f0));
-  const float2 r1 = f2_unpack(f2_fma(a2, f2_sub(f2_pack(fx[2], fx[3]), f1), f1));
+  const float2 r0 = f2_unpack(f2_add(f0, f2_mul(a2, f2_sub(f2_pack(fx[0], fx[1]), f0))));
+  const float2 r1 = f2_unpack(f2_add(f1, f2_mul(a2, f2_sub(f2_pack(fx[2], fx[3]), f1))));
   return Vec<float>{{r0.x, r0.y, r1.x, r1.y}};
 }
 
@@ -113,12 +115,14 @@ split_kernel(const __grid_constant__ SplitArgs sa) {
     return;
   const size_t sbytes = stage_bytes<T>(gm.stage_elems);
   SplitShared& sh = *reinterpret_cast<SplitShared*>(smem + NS * sbytes);
-  T* const srow = reinterpret_cast<T*>(&sh + 1);  // FP32: source factors; both: collision factors
+  // FP32: source factors of the rows, FP64: 1 - |c_x| (or half); both: collision factors
+  T* const srow = reinterpret_cast<T*>(&sh + 1);
   T* const m1 = srow + kMaxTileRows;
   T* const scol = reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(m1 + kMaxTileRows) + 15) & ~(uintptr_t)15);
   T* const m2 = scol + pitch;
   for (int r = tid; r < rows; r += NT) {
-    if (sizeof(T) == 4) srow[r] = (T)a.tab.srow32[i0 + r];
+    srow[r] = sizeof(T) == 4 ? (T)a.tab.srow32[i0 + r]
+                             : (T)(1.0 - (STRANG ? 0.5 : 1.0) * fabs(a.tab.cx[i0 + r]));
     if (BGK) m1[r] = sizeof(T) == 8 ? (T)a.tab.m1[i0 + r] : (T)a.tab.m1_32[i0 + r];
   }
   for (int j = tid; j < pitch; j += NT) {
@@ -267,17 +271,9 @@ split_kernel(const __grid_constant__ SplitArgs sa) {
   // one warp: fold the warps' sums of plane k (slot b) and store them
   auto fold = [&](int k, int b) {
     const float2 x = sh.wn[b][lane % NW];
-    double n;
-    if constexpr (sizeof(T) == 4) {
-      float f = x.x;
+    double n = sizeof(T) == 4 ? (double)x.x : (double)x.x + (double)x.y;
 #pragma unroll
-      for (int o = NW / 2; o > 0; o >>= 1) f += __shfl_down_sync(0xffffffffu, f, o);
-      n = (double)f;
-    } else {
-      n = (double)x.x + (double)x.y;
-#pragma unroll
-      for (int o = NW / 2; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
-    }
+    for (int o = NW / 2; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
     if (lane == 0) a.part.n[(size_t)k * nt + t] = n;
   };
   // one warp: the outflow of g (plane k, in the stage at sb) through the
@@ -324,7 +320,7 @@ split_kernel(const __grid_constant__ SplitArgs sa) {
         if (NT * m >= nvec) break;
         T* const c = sb + offset(m);
         const Vec<T> own = *reinterpret_cast<const Vec<T>*>(c);
-        const Vec<T> g = x_step_vec(own, xr[m], ax[m]);
+        const Vec<T> g = x_step_vec(own, xr[m], ax[m], sizeof(T) == 8 ? srow[row_of(m)] : (T)0);
         if (flg >> m & 1) *reinterpret_cast<Vec<T>*>(c) = g;
 #pragma unroll
         for (int e = 0; e < VEC; e++) xr[m][e] = own.e[e];
@@ -347,7 +343,7 @@ split_kernel(const __grid_constant__ SplitArgs sa) {
               u = wall_inflow(ih, v * VEC);
             o = *reinterpret_cast<const Vec<T>*>(hrow + v * VEC);
 #pragma unroll
-            for (int e = 0; e < VEC; e++) o.e[e] = x_step(o.e[e], u.e[e], axh);
+            for (int e = 0; e < VEC; e++) o.e[e] = x_step(o.e[e], u.e[e], axh, (T)1 - axh);
           }
           *reinterpret_cast<Vec<T>*>(hrow + v * VEC) = o;
         }
@@ -455,7 +451,8 @@ split_kernel(const __grid_constant__ SplitArgs sa) {
         if constexpr (STRANG) {
           if (ANY && edge && in) *reinterpret_cast<Vec<T>*>(static_cast<T*>(sa.h_wall) + (size_t)i0 * pitch + so) = out;
           const Vec<T> h = out;
-          if (!ANY || !deferred) out = x_step_vec(h, hr[m], ax[m]);
+          if (!ANY || !deferred)
+            out = x_step_vec(h, hr[m], ax[m], sizeof(T) == 8 ? srow[row_of(m)] : (T)0);
 #pragma unroll
           for (int e = 0; e < VEC; e++) hr[m][e] = h.e[e];
         }
@@ -624,7 +621,7 @@ __global__ void __launch_bounds__(kWallThreads) strang_wall_kernel(const __grid_
     for (int e = 0; e < VEC; e++) {
       double g = gsee * gse[e];
       if (refl > 0.0) g = fma(refl, (double)mir.e[e], g);
-      o.e[e] = x_step(o.e[e], (T)g, (T)0.5 * cx);
+      o.e[e] = x_step(o.e[e], (T)g, (T)0.5 * cx, (T)1 - (T)0.5 * cx);
       const T s = sum + o.e[e], b = s - sum;  // TwoSum
       err += (sum - (s - b)) + (o.e[e] - b);
       sum = s;
