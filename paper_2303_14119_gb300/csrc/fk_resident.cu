@@ -109,7 +109,11 @@ struct FinShared {
   double wall[3];   // Gamma_pe, Gamma_see, Gamma_vac of the new state
   double off, n;    // densities below this block; of all planes
   double sigma;     // sigma of the new state
-  int stop, bad;
+  // stop: the step's inputs are void, leave before it; end: this block found a
+  // fault in the new state, leave after the step.  Two words: end is read after
+  // the step's last barrier, when thread 0 may already be setting stop for the
+  // next one.
+  int stop, end, bad;
   DevState d;       // block 0: the run's scalars
 };
 
@@ -132,7 +136,7 @@ __device__ __forceinline__ void resident_finalize(const ResidentArgs& ra, const 
   if (t == 0) {
     sh.d = *st;
     sh.sigma = advance_sigma(sh.d.sigma, dt, sh.d.g_see, sh.d.g_pe, refl);
-    sh.stop = sh.bad = 0;
+    sh.stop = sh.end = sh.bad = 0;
   }
   fin_sync();
   for (int step = 0; step < ra.rs.n_steps; step++) {
@@ -258,7 +262,7 @@ __device__ __forceinline__ void resident_finalize(const ResidentArgs& ra, const 
         bad |= kFlagNumeric;
       if (bad) atomicOr(&st->flags, bad);
       count_arrival(ra.rs.go, bad ? 1u + kGoStop : 1u);
-      sh.stop = bad != 0;
+      sh.end = bad != 0;
     }
     // ---- while the units march on: what only the getters and the ledger read
     if (live) {
@@ -307,7 +311,7 @@ __device__ __forceinline__ void resident_finalize(const ResidentArgs& ra, const 
     }
     if (t == 0) sh.sigma = advance_sigma(sh.sigma, dt, sh.wall[1], sh.wall[0], refl);
     fin_sync();
-    if (sh.stop) return;
+    if (sh.end) return;
   }
 }
 

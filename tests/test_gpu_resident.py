@@ -13,7 +13,7 @@ import numpy as np
 import pytest
 
 import oracle
-from oracle import QE
+from oracle import ME, QE
 from paper_2303_14119_gb300 import fk
 
 from test_gpu_parity import make_pair, rel_l1, strong_physics
@@ -157,3 +157,39 @@ def test_courant_bound_freezes_at_the_same_step(prec):
     assert np.array_equal(fa, fb)
     for g in pair:
         g.close()
+
+
+@pytest.mark.parametrize("shape", [(60, 32, 28), (300, 32, 28), (417, 96, 72)])
+def test_flag_raised_by_a_unit_during_a_launch(shape):
+    """A value below zero reaches the wall in step 38 of a launch: the unit that
+    sees it raises the flag, every finalize CTA leaves before that step, and
+    the state is that of step 37, as with single launches.  (Courant numbers
+    that sum to 1 + 5e-13, within the bound, give the fastest row a weight of
+    -5e-13 for its own value: what left plane 37 arrives with weights c_x^37,
+    and a step later with the negative one.)"""
+    nx, nv1, nv2 = shape
+    far, states = 37, []
+    for form in ("launches of many steps", "single launches", "the steps before"):
+        g = fk.Grid(nx, nv1, nv2, 20e-6, -6e7, 6e7, -3e7, 3e7, cfl=0.5, precision=fk.FK_F64)
+        info = g.info()
+        c2 = 1.0 - 0.5 * (1.0 - 1.0 / nv1) + 5e-13
+        g.set_fields(-c2 * info["dv2"] / info["dt"] * ME / QE, False, 0.0)
+        f0 = np.zeros(shape)
+        f0[far, 0, 3] = 1.0
+        g.set_f(f0)
+        if form == "single launches":
+            g.set_kernel_timing(True)
+        g.step(far if form == "the steps before" else 100)
+        ok = form == "the steps before"
+        assert fk.fk_sync_status(g.h) == (fk.FK_OK if ok else fk.FK_ENEGATIVE)
+        f = np.empty(shape)
+        if ok:
+            g.get_f(f)
+        else:
+            with pytest.raises(fk.FkError):
+                g.get_f(f)
+        states.append(f)
+        g.close()
+    assert states[2][0, 0, 3] > 0
+    assert np.array_equal(states[0], states[1])
+    assert np.array_equal(states[0], states[2])
