@@ -261,6 +261,11 @@ __device__ __forceinline__ void resident_finalize(const ResidentArgs& ra, const 
                        !isfinite(ntot) || !isfinite(sh.sigma)))
         bad |= kFlagNumeric;
       if (bad) atomicOr(&st->flags, bad);
+      // A fault of this block's planes is known to this block alone: the units
+      // learn of it through go, the other blocks, which wait for the next
+      // step's arrivals, through arrive (every one of them has passed this
+      // step's, or the exchange would not have ended).
+      if (bad) count_arrival(ra.rs.arrive, kGoStop);
       count_arrival(ra.rs.go, bad ? 1u + kGoStop : 1u);
       sh.end = bad != 0;
     }

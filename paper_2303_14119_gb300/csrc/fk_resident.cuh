@@ -9,7 +9,7 @@ namespace fk {
 // finalize CTAs that its planes are done and waits for the coefficients of
 // the new state.  Both counters start at kCountZero.
 struct Resident {
-  unsigned* arrive;  // one count per unit and step
+  unsigned* arrive;  // one count per unit and step; kGoStop: no further step
   unsigned* go;      // n_fin counts per step; kGoStop: no further step
   unsigned n_units;
   unsigned n_fin;    // finalize CTAs

@@ -8,6 +8,7 @@ rows, one and several finalize blocks, collisions and reflection, and with an
 E_x that changes its sign along x and in time (the planes fetched ahead of a
 step were then laid out for the other v1 neighbour)."""
 import os
+import time
 
 import numpy as np
 import pytest
@@ -193,3 +194,82 @@ def test_flag_raised_by_a_unit_during_a_launch(shape):
     assert states[2][0, 0, 3] > 0
     assert np.array_equal(states[0], states[1])
     assert np.array_equal(states[0], states[2])
+
+
+def lower_fields_and_go_on(pair, shape):
+    """Fields within the bound clear the error; both forms step on alike."""
+    for g in pair:
+        g.set_fields(0.0, False, 0.0)
+        assert fk.fk_sync_status(g.h) == fk.FK_OK
+        g.step(20)
+        g.sync()
+    assert_same(*pair)
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+@pytest.mark.parametrize("nx", [131, 300, 417])
+@pytest.mark.parametrize("where", ["first block", "last block"])
+def test_courant_stop_found_by_one_finalize_block(prec, nx, where):
+    """|c_1| grows past the bound in one block's planes only, at the wall (the
+    surface charges) or in the last plane (the space charge of a source there
+    grows): the other finalize CTAs stop with it at once, the status is the
+    Courant one, and lower fields bring the grid back."""
+    shape, h = (nx, 32, 28), 20e-6
+    pair = []
+    for _ in range(2):
+        g, o = make_pair(shape, prec=prec)
+        f0, sigma = strong_physics(g, o, shape, seed=11)
+        if where == "first block":
+            g.set_see(9.0, 400.0, 1.0, 400.0)
+            sigma *= 2.0
+        else:
+            g.set_source(1e13 * (nx / 300) ** 2, 0.9 * h, h, 300.0)
+            f0[:], sigma = 0.0, 0.0
+        g.set_state(f0, sigma)
+        pair.append(g)
+    a, b = pair
+    b.set_kernel_timing(True)
+    states = []
+    for g in pair:
+        g.step(100)
+        t = time.perf_counter()
+        assert fk.fk_sync_status(g.h) == fk.FK_ECFL
+        assert time.perf_counter() - t < 0.5  # no wait ran out
+        f = np.empty(shape)
+        with pytest.raises(fk.FkError):
+            g.get_f(f)
+        states.append(f)
+    assert np.array_equal(*states)
+    lower_fields_and_go_on(pair, shape)
+    ex = a.history(200)[:, 7]
+    assert 30 < len(ex) - 21 < 70  # the step of the stop, by the oracle 39 to 55
+    for g in pair:
+        g.close()
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+@pytest.mark.parametrize("nx", [60, 131, 417])
+def test_non_finite_stop_of_several_finalize_blocks(prec, nx):
+    """A plane whose sum overflows in the step's partial sums (FP32 sums of FP32
+    grids; FP64 grids take values below 2^128): block 0 finds it, and every
+    finalize CTA leaves with the non-finite status, not a timeout."""
+    shape = (nx, 32, 28)
+    f0 = np.zeros(shape)
+    f0[nx // 2, :, ::4] = 1e38 if prec == fk.FK_F32 else 1e40
+    states = []
+    for single in (False, True):
+        g = make_pair(shape, prec=prec)[0]
+        g.set_fields(-1e5, False, 0.0)
+        g.set_f(f0)
+        assert fk.fk_sync_status(g.h) == fk.FK_OK
+        g.set_kernel_timing(single)
+        g.step(40)
+        t = time.perf_counter()
+        assert fk.fk_sync_status(g.h) == fk.FK_ENUMERIC
+        assert time.perf_counter() - t < 0.5
+        f = np.empty(shape)
+        with pytest.raises(fk.FkError):
+            g.get_f(f)
+        states.append(f)
+        g.close()
+    assert np.array_equal(*states)
