@@ -80,6 +80,13 @@ __device__ __forceinline__ double take_value(const unsigned long long* p, long l
   return __longlong_as_double((long long)v);
 }
 
+// The exchange's rows of kFinMaxBlocks slots: two for the densities (even and
+// odd steps), then three for the velocity-edge sums.
+constexpr int kXchRows = 5;
+__device__ __forceinline__ unsigned long long* lv_slots(const ResidentArgs& ra, int step) {
+  return ra.xch + (size_t)(2 + step % 3) * kFinMaxBlocks;
+}
+
 // sum over tiles of plane k's partials, in tile order (as finalize_body)
 __device__ __forceinline__ double plane_sum(const double* p, int nu) {
   double s = 0.0;
@@ -195,7 +202,13 @@ __device__ __forceinline__ void resident_finalize(const ResidentArgs& ra, const 
       if (w == 0) {
         if (lane == 0) {
           put_value(slot + blk, btot);
+          // this block's slots of the next step, emptied before this step's
+          // release of go, which orders that before any read in the next one.
+          // The last reads of those slots lie before a go that this block has
+          // seen the units pass: a step back for the densities, read before it;
+          // two for the velocity-edge sums, read after it (a third row).
           st_relaxed64(ra.xch + (size_t)((step + 1) & 1) * kFinMaxBlocks + blk, kNoValue);
+          st_relaxed64(lv_slots(ra, step + 1) + blk, kNoValue);
         }
         bool ok = true;
         const double b0 = lane < n_fin ? take_value(slot + lane, lim, &ok) : 0.0;
@@ -283,11 +296,8 @@ __device__ __forceinline__ void resident_finalize(const ResidentArgs& ra, const 
       l = warp_tree(l, kFinThreads / 32);
       bool ok = true;
       if (n_fin > 1) {
-        unsigned long long* slot = ra.xch + (size_t)(2 + (step & 1)) * kFinMaxBlocks;
-        if (lane == 0) {
-          put_value(slot + blk, l);
-          st_relaxed64(ra.xch + (size_t)(2 + ((step + 1) & 1)) * kFinMaxBlocks + blk, kNoValue);
-        }
+        unsigned long long* slot = lv_slots(ra, step);
+        if (lane == 0) put_value(slot + blk, l);
         if (blk == 0)
           l = (lane < n_fin ? take_value(slot + lane, lim, &ok) : 0.0) +
               (lane + 32 < n_fin ? take_value(slot + lane + 32, lim, &ok) : 0.0);
@@ -384,7 +394,7 @@ int fit_sized(int optin, size_t smem, bool padded) {
 
 // two 32-bit counters, each on its own 128-byte line, then the exchange
 constexpr int kXchWord = 64;
-int resident_scratch_words() { return kXchWord + 2 * 4 * kFinMaxBlocks; }
+int resident_scratch_words() { return kXchWord + 2 * kXchRows * kFinMaxBlocks; }
 
 size_t resident_smem_bytes(int precision, const Geom& gm, int pitch) {
   // a unit's block without the argument slot of the batched kernels, with

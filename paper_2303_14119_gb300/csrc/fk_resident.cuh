@@ -24,7 +24,7 @@ struct ResidentArgs {
   StepArgs a;   // step 0's; odd steps swap f_in and f_out
   FinOut o;
   Resident rs;
-  unsigned long long* xch;  // [4][finalize CTAs] exchange of block sums, all bits set
+  unsigned long long* xch;  // [rows][kFinMaxBlocks] exchange of block sums, all bits set
 };
 
 // Words of the block that holds a launch's counters and exchange slots; every

@@ -273,3 +273,29 @@ def test_non_finite_stop_of_several_finalize_blocks(prec, nx):
         states.append(f)
         g.close()
     assert np.array_equal(*states)
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+@pytest.mark.parametrize("nx", [129, 4096, 4225, 8192])
+def test_exchange_of_many_finalize_blocks(prec, nx):
+    """2, 32, 34 and 64 finalize CTAs, over launches of 1 to 5 and 128 steps (the
+    rows of the exchange in every order): the ledger, whose velocity-edge loss
+    goes through it after the step, and all the rest equal single launches."""
+    shape = (nx, 6, 8)
+    pair = []
+    for _ in range(2):
+        g, o = make_pair(shape, prec=prec)
+        f0, sigma = strong_physics(g, o, shape, seed=nx, c1f=0.08)
+        g.set_state(f0, sigma)
+        pair.append(g)
+    a, b = pair
+    b.set_kernel_timing(True)
+    for n in (1, 2, 3, 4, 5, 128):
+        a.step(n)
+        b.step(n)
+    a.sync()
+    b.sync()
+    assert a.ledger()["lv"] > 0
+    assert_same(a, b)
+    a.close()
+    b.close()
