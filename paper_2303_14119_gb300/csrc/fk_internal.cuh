@@ -238,6 +238,15 @@ cudaError_t launch_convert(const void* src, void* dst, size_t rows, int nv2, int
 
 enum FinalizeMode { kModeStep = 0, kModeRefresh = 1, kModeReset = 2 };
 
+// Whether a value is below zero, as x < 0 has it (false for a NaN of either
+// sign), without an FP64 comparison: the bits of the negative numbers run from
+// the one after -0 to -infinity's, and those of the NaN with the sign bit follow.
+__device__ __forceinline__ bool is_negative(float x) { return x < 0.f; }
+__device__ __forceinline__ bool is_negative(double x) {
+  return (unsigned long long)__double_as_longlong(x) - 0x8000000000000001ull <=
+         0x7FEFFFFFFFFFFFFFull;
+}
+
 // Error text for calls without a grid (read back by fk_last_error(NULL)).
 void set_thread_error(const char* msg);
 

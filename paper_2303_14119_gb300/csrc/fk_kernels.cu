@@ -404,13 +404,6 @@ cudaError_t launch_step_pass(const StepArgs& a, int precision, int mode, cudaStr
 // evaluations of a grid set to a new point of a scan are 460 us shorter.
 constexpr int kMomThreads = 256;
 
-// a state has to hold no value below zero
-__device__ __forceinline__ bool below_zero(float x) { return x < 0.f; }
-__device__ __forceinline__ bool below_zero(double x) {
-  const int h = __double2hiint(x);
-  return h < 0 && ((h << 1) | __double2loint(x)) != 0;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_constant__ StepArgs a) {
   __shared__ double sh[32];
@@ -441,7 +434,7 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_const
         x[2 * j + 1] = d.y;
       }
 #pragma unroll
-      for (int q = 0; q < kGroup; q++) neg |= below_zero(x[q]);
+      for (int q = 0; q < kGroup; q++) neg |= is_negative(x[q]);
       acc.s = add_group(x, acc.s);
     } else {
 #pragma unroll
@@ -449,7 +442,7 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_const
         const float x[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
 #pragma unroll
         for (int e = 0; e < 4; e++) {
-          neg |= below_zero(x[e]);
+          neg |= is_negative(x[e]);
           acc.add(x[e]);
         }
       }

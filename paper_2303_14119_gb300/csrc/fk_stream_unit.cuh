@@ -314,13 +314,6 @@ struct ItemVals {
   float pad;
 };
 
-// whether a value is below zero, without an FP64 comparison
-__device__ __forceinline__ bool is_negative(float x) { return x < 0.f; }
-__device__ __forceinline__ bool is_negative(double x) {
-  const int hi = __double2hiint(x);
-  return hi < 0 && ((hi << 1) | __double2loint(x)) != 0;
-}
-
 // Wall (x = 0, v1 < 0: Eqs. 12-14) or vacuum (x = h_max, v1 > 0) sums of
 // f^{n+1} over this consumer thread's cells of one plane, read back from
 // its own stores; returns whether one of those cells is negative.  Called

@@ -149,3 +149,25 @@ def test_every_allocation_failure_of_a_creation_is_reported(prec, monkeypatch):
     for x in grids + [g]:
         x.step(2)
         x.close()
+
+
+@pytest.mark.parametrize("prec", [fk.FK_F64, fk.FK_F32])
+@pytest.mark.parametrize("plane", [0, 5, 11])
+@pytest.mark.parametrize("value, status", [
+    (np.nan, fk.FK_ENUMERIC), (np.copysign(np.nan, -1.0), fk.FK_ENUMERIC),
+    (np.inf, fk.FK_ENUMERIC), (-np.inf, fk.FK_ENEGATIVE), (-0.0, fk.FK_OK),
+    (-1e-30, fk.FK_ENEGATIVE)])
+def test_input_values_that_are_no_numbers(prec, plane, value, status):
+    """A NaN of either sign is not a negative value: x86 makes its own with the
+    sign bit set."""
+    shape = (12, 16, 20)
+    g, o = make_pair(shape, prec=prec)
+    f0, sigma = strong_physics(g, o, shape, seed=33, c1f=0.05)
+    f0[plane, 3, 6] = value
+    if status == fk.FK_OK:
+        g.set_f(f0)
+    else:
+        with pytest.raises(fk.FkError) as ei:
+            g.set_f(f0)
+        assert ei.value.status == status
+    g.close()
