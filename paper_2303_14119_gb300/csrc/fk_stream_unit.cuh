@@ -531,9 +531,12 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
   // variant); elsewhere the pointers stay in registers (measured faster)
   constexpr bool SAU = SA && (NT == kHalfThreads || BGK);
   // compact index arithmetic (an item's plane in one multiply-add, 32-bit
-  // stage and plane sizes): faster in the half-unit, padded-row and
-  // collision variants, 1 % slower in the plain whole-CTA one (measured)
-  constexpr bool COMPACT = NT == kHalfThreads || PADDED || BGK;
+  // stage and plane sizes), where it keeps the march's registers within the
+  // launch bounds: without it the plain whole-CTA FP32 batch kernel spills 40
+  // bytes in the march, and three grids of 1024 x 256 x 256 take 318 us a
+  // launch instead of 263 (0.745 and 0.90 of copy bandwidth).  The FP64 and the
+  // resident plain whole-CTA kernels spill less without it.
+  constexpr bool COMPACT = NT == kHalfThreads || PADDED || BGK || (!RES && sizeof(T) == 4);
   using StageSz = std::conditional_t<COMPACT, unsigned, size_t>;  // < 227 KB
   using PlaneSz = std::conditional_t<COMPACT, int, size_t>;
   const Geom& gm = a.geom;
