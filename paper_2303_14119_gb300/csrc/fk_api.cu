@@ -10,6 +10,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -29,6 +30,8 @@ constexpr int kGraphSteps = 32;  // steps per captured graph (even)
 // sums in its last one cost, in planes (5 and 7 us a launch-step against 1.5
 // us a plane at 321 x 117 x 117; more than 2 left the other chunks too long)
 constexpr int kResidentFirst = 2, kResidentLast = 2;
+// turns that resident launches of grids of less than half the GPU may take
+constexpr double kSmallTurns = 3.0;
 constexpr int kMaxTimed = 8192;  // step-kernel launches timed between reads
 constexpr size_t kStageElems = size_t(1) << 23;  // FP64 staging chunk, 64 MB
 
@@ -111,9 +114,72 @@ fk_status upload_params(fk_grid* g) {
   return FK_OK;
 }
 
+struct Flights {
+  std::mutex m;
+  InFlight* first = nullptr;
+  long long clock = 0;
+};
+Flights& flights() {
+  static Flights* f = new Flights();  // grids may outlive the process's static objects
+  return *f;
+}
+
+}  // namespace
+
+void fk::note_queued(InFlight* f, int dev, cudaStream_t stream, double share) {
+  Flights& a = flights();
+  std::lock_guard<std::mutex> lock(a.m);
+  f->dev = dev;
+  f->stream = stream;
+  f->share = share;
+  // others count while they were queued after this one's last wait: what was
+  // left alone for longer has most likely finished
+  auto beside = [&](const InFlight* q) {
+    return q != f && q->dev == dev && q->stream != stream && q->queued_at > f->idle_at;
+  };
+  double sum = share, widest = share;
+  for (const InFlight* q = a.first; q; q = q->next)
+    if (beside(q)) {
+      sum += q->share;
+      widest = std::max(widest, q->share);
+    }
+  const double load = widest < 0.5 ? sum / kSmallTurns : sum;
+  f->load = std::max(f->load, load);
+  for (InFlight* q = a.first; q; q = q->next)
+    if (beside(q)) q->load = std::max(q->load, load);
+  f->queued_at = ++a.clock;
+  if (!f->queued) {
+    f->queued = true;
+    f->prev = nullptr;
+    f->next = a.first;
+    if (a.first) a.first->prev = f;
+    a.first = f;
+  }
+}
+
+void fk::note_idle(InFlight* f) {
+  Flights& a = flights();
+  std::lock_guard<std::mutex> lock(a.m);
+  f->idle_at = a.clock;
+  if (!f->queued) return;
+  f->queued = false;
+  f->last_load = f->load;
+  f->load = 0;
+  if (f->prev)
+    f->prev->next = f->next;
+  else
+    a.first = f->next;
+  if (f->next) f->next->prev = f->prev;
+  f->prev = f->next = nullptr;
+}
+
+double fk::load_beside(InFlight* f) {
+  std::lock_guard<std::mutex> lock(flights().m);
+  return std::max(f->load, f->last_load);
+}
+
 // Synchronise, read the device scalars, and re-base the buffer bookkeeping
 // on the last valid state.
-}  // namespace
 
 fk_status fk::sync_state(fk_grid* g, DevState* out) {
   return sync_state_with(g, out, nullptr, nullptr);
@@ -130,6 +196,7 @@ fk_status fk::sync_state_with(fk_grid* g, DevState* out, double* n_e, double* Ex
   if (n_e) FK_CUDA(g, cudaMemcpyAsync(hv, g->d_ne, vb, cudaMemcpyDeviceToHost, g->stream));
   if (Ex) FK_CUDA(g, cudaMemcpyAsync(hv + g->nx, g->d_Ex, vb, cudaMemcpyDeviceToHost, g->stream));
   FK_CUDA(g, cudaStreamSynchronize(g->stream));
+  note_idle(&g->flight);
   *out = *hst;
   if (n_e) memcpy(n_e, hv, vb);
   if (Ex) memcpy(Ex, hv + g->nx, vb);
@@ -325,12 +392,27 @@ cudaError_t enqueue_step(fk_grid* g, int cur, cudaStream_t s, cudaEvent_t ev0, c
 }
 
 // Whether fk_step runs on the resident step kernel: the unsplit scheme on
-// streaming tiles, at every size (it was the faster one from 64 x 48 x 48 to
-// 1024 x 256 x 256, in both storage types; figures in fk_resident.cu).  (A withheld pipeline item, a test knob, has to lie in the
-// first step of the unit it names.)
-bool use_resident(const fk_grid* g) {
-  return g->use_stream && g->scheme == kSchemeUnsplit && g->res_chunks > 0 &&
-         g->prm.withhold_item < g->res_chunk_len - g->res_chunk_off;
+// streaming tiles, at every size and from one step a call on (us a step, single
+// launches -> resident, calls of 1 and of 128 steps: 64 x 48 x 48 FP64 38.9 ->
+// 22.3 and 34.9 -> 15.9; 321 x 117 x 117 FP32 28.7 -> 28.7 and 26.2 -> 21.6;
+// 1024 x 256 x 256 FP32 115.1 -> 114.8 and 109.7 -> 105.6), unless grids on other
+// streams step at the same time and the CTAs of all do not fit the GPU: resident
+// launches would then take turns (four grids of 321 x 117 x 117 FP32 on their
+// own streams: 84 us a step of all, single launches 40; of 64 x 48 x 48 FP64,
+// which fit: 17 and 35).  Where every one takes less than half of the GPU, whose
+// single launches are mostly gaps, up to three turns still pay (twelve of 64 x
+// 48 x 48 FP32, calls of 16 and of 128 steps: 34 and 32 us, single launches 67
+// and 37; sixteen: 44 and 43, 82 and 38).  A captured call stays resident: a
+// graph cannot be replayed into a capture.  (A withheld pipeline item, a test knob, has to lie
+// in the first step of the unit it names.)
+bool use_resident(fk_grid* g) {
+  if (!g->use_stream || g->scheme != kSchemeUnsplit || g->res_chunks <= 0 ||
+      g->prm.withhold_item >= g->res_chunk_len - g->res_chunk_off)
+    return false;
+  if (load_beside(&g->flight) <= 1.0) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(g->stream, &cap) == cudaSuccess &&
+         cap != cudaStreamCaptureStatusNone;
 }
 
 // Calls that change a grid's state are refused while a batch steps it.
@@ -387,6 +469,7 @@ fk_status refresh(fk_grid* g, bool tables) {
 
 void free_grid(fk_grid* g) {
   if (!g) return;
+  note_idle(&g->flight);
   cudaSetDevice(g->dev);
   if (g->stream) cudaStreamSynchronize(g->stream);
   for (int p = 0; p < 2; p++)
@@ -483,6 +566,7 @@ fk_status build_graph(fk_grid* g, int parity) {
 // fit the GPU at once beside the launch's finalize CTAs.
 void plan_resident(fk_grid* g, int sms) {
   g->res_chunks = g->res_chunk_len = 0;
+  g->res_share = 1.0;
   if (!g->use_stream) return;
   const int per_sm = resident_ctas_per_sm(g->prec, g->geom, g->pitch, g->pitch != g->nv2);
   const int slots = sms * per_sm - finalize_blocks(g->nx);
@@ -496,6 +580,7 @@ void plan_resident(fk_grid* g, int sms) {
   g->res_chunk_len = len;
   g->res_chunk_off = first;
   g->res_chunks = (g->nx + g->res_chunk_off + len - 1) / len;
+  g->res_share = (double)(g->geom.n_tiles * g->res_chunks + finalize_blocks(g->nx)) / (sms * per_sm);
 }
 
 // Tiles of v1 rows (never straddling the sign change of v1) and chunks of
@@ -921,6 +1006,7 @@ fk_status fk_step(fk_grid* g, int64_t n) {
   if (g->known_flags) return flags_status(g, g->known_flags);
   FK_CUDA(g, cudaSetDevice(g->dev));
   while (n > 0) {
+    note_queued(&g->flight, g->dev, g->stream, g->res_share);
     if (g->timing) {
       const bool rec = g->ev_used < kMaxTimed;
       FK_CUDA(g, enqueue_step(g, g->enq_cur, g->stream, rec ? g->ev[2 * g->ev_used] : nullptr,

@@ -88,6 +88,7 @@ struct fk_batch {
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t fin_ev = nullptr;   // the batch's work up to an enqueue
   cudaEvent_t pending = nullptr;  // the last gather, not yet waited for
+  InFlight flight;
   std::string err;
 };
 
@@ -396,6 +397,7 @@ fk_status enqueue_steps(fk_batch* b, long long n) {
 // Release the grids (re-based on their device step counters) and free.
 void free_batch(fk_batch* b) {
   if (!b) return;
+  note_idle(&b->flight);
   cudaSetDevice(b->dev);
   if (b->stream) cudaStreamSynchronize(b->stream);
   if (b->copy_stream) cudaStreamSynchronize(b->copy_stream);  // a gather or copy in flight
@@ -437,6 +439,7 @@ fk_status read_states(fk_batch* b, std::vector<const DevState*>* st) {
     (*st)[i] = static_cast<const DevState*>(g->h_stage);
   }
   BK_CUDA(b, cudaStreamSynchronize(b->stream));
+  note_idle(&b->flight);
   return FK_OK;
 }
 
@@ -556,6 +559,7 @@ fk_status fk_batch_step(fk_batch* b, int64_t n) {
   const NvtxRange range("fk_batch_step");
   if (n < 0) return bfail(b, FK_EINVAL, "n must be >= 0");
   BK_CUDA(b, cudaSetDevice(b->dev));
+  if (n > 0) note_queued(&b->flight, b->dev, b->stream, 1.0);  // a batch fills the GPU
   return enqueue_steps(b, n);
 }
 
@@ -610,6 +614,7 @@ fk_status fk_batch_moments(fk_batch* b, double* sigma, double* gamma_pe, double*
     if (Ex) BK_CUDA(b, cudaMemcpyAsync(hv + g->nx, g->d_Ex, vb, cudaMemcpyDeviceToHost, b->stream));
   }
   BK_CUDA(b, cudaStreamSynchronize(b->stream));
+  note_idle(&b->flight);
   size_t off = 0;
   for (int i = 0; i < b->n; i++) {
     fk_grid* g = b->grids[i];

@@ -9,6 +9,29 @@
 
 #include "fk_internal.cuh"
 
+namespace fk {
+// The steps that a grid's or a batch's stream may still hold (from the enqueue
+// to the next wait for the stream), linked with the others' of the process under
+// one lock.  A resident launch holds its CTAs' places on the GPU for many steps,
+// so launches of grids on several streams run side by side only where their CTAs
+// all fit; where they do not, single steps share the GPU better (fk_step).
+struct InFlight {
+  int dev = 0;
+  cudaStream_t stream = nullptr;
+  double share = 0;      // of the GPU's places for resident CTAs
+  long long queued_at = 0, idle_at = 0;  // counts of the process's enqueues
+  // the largest sum of shares on the device while steps of this one were queued
+  // beside others' (above 1: resident launches would take too many turns): since
+  // the last wait, and between the two waits before it
+  double load = 0, last_load = 0;
+  InFlight *prev = nullptr, *next = nullptr;
+  bool queued = false;
+};
+void note_queued(InFlight* f, int dev, cudaStream_t stream, double share);
+void note_idle(InFlight* f);
+double load_beside(InFlight* f);
+}  // namespace fk
+
 struct fk_grid {
   int dev = 0;
   cudaStream_t stream = nullptr;
@@ -34,6 +57,8 @@ struct fk_grid {
   // resident step kernel: x-chunks of its units (0 chunks: this grid does not
   // use it), its counters and the velocity-edge partials of its odd steps
   int res_chunk_len = 0, res_chunk_off = 0, res_chunks = 0;
+  double res_share = 1.0;  // its CTAs' share of those that fit the GPU at once
+  fk::InFlight flight;
   unsigned* d_res = nullptr;
   double* d_lv_odd = nullptr;
   int part_cap = 0;   // tiles the partial-sum buffers hold

@@ -8,6 +8,7 @@ rows, one and several finalize blocks, collisions and reflection, and with an
 E_x that changes its sign along x and in time (the planes fetched ahead of a
 step were then laid out for the other v1 neighbour)."""
 import os
+import threading
 import time
 
 import numpy as np
@@ -299,3 +300,86 @@ def test_exchange_of_many_finalize_blocks(prec, nx):
     assert_same(a, b)
     a.close()
     b.close()
+
+
+def stepped_alone(shapes, precs, steps):
+    out = []
+    for shape, prec in zip(shapes, precs):
+        g, o = make_pair(shape, prec=prec)
+        f0, sigma = strong_physics(g, o, shape, seed=5, c1f=0.08)
+        g.set_state(f0, sigma)
+        g.step(steps)
+        g.sync()
+        out.append(g)
+    return out
+
+
+def test_grids_on_their_own_streams_from_several_threads():
+    """Grids of several sizes, each on its own stream and thread, some of them
+    beside a batch: whichever form their steps take meanwhile, the states are
+    those of each grid stepped alone."""
+    shapes = [(321, 117, 61), (64, 48, 48), (200, 96, 72), (300, 40, 45), (64, 48, 48)]
+    precs = [fk.FK_F32, fk.FK_F64, fk.FK_F32, fk.FK_F64, fk.FK_F32]
+    alone = stepped_alone(shapes, precs, 300)
+    grids = stepped_alone(shapes, precs, 0)
+    members = stepped_alone([(128, 64, 64)] * 2, [fk.FK_F32] * 2, 0)
+    errors = []
+
+    def work(step, sync):
+        try:
+            for n in (1, 33, 130, 7, 64, 65):  # 300 in all
+                step(n)
+                sync()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    with fk.Batch(members) as b:
+        threads = [threading.Thread(target=work, args=(x.step, x.sync)) for x in grids + [b]]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    assert not errors
+    for a, g in zip(alone, grids):
+        assert_same(a, g)
+    for g in alone + grids + members:
+        g.close()
+
+
+def test_grids_on_their_own_streams_share_the_gpu():
+    """Four grids that do not fill the GPU's time alone (their steps are bound by
+    latency) take less together than one after the other: resident launches,
+    which would take turns, give way.  The bound is far from both sides (0.97 of
+    the sum when they take turns, about 0.5 side by side)."""
+    shape = (321, 117, 117)
+    grids = stepped_alone([shape] * 4, [fk.FK_F32] * 4, 0)
+    for g in grids:
+        g.set_fields(-1e5, False, 0.0)  # the Courant numbers stay what they are
+        g.step(64)
+        g.sync()
+
+    def best(run):
+        times = []
+        for _ in range(6):
+            t = time.perf_counter()
+            run()
+            times.append(time.perf_counter() - t)
+        return min(times)
+
+    def in_turn():
+        for g in grids:
+            g.step(256)
+            g.sync()
+
+    def together():
+        for g in grids:
+            g.step(256)
+        for g in grids:
+            g.sync()
+
+    apart = best(in_turn)
+    assert best(together) < 0.75 * apart
+    # and back: one after the other again, in the resident form
+    assert best(in_turn) < 1.2 * apart
+    for g in grids:
+        g.close()
