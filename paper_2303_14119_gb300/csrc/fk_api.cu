@@ -297,11 +297,16 @@ fk_status evaluate(fk_grid* g, int mode) {
   return FK_OK;
 }
 
+// The tiles of a scheme's fused split step (none: it runs as passes).
+const Geom& split_plan(const fk_grid* g, int scheme) {
+  return g->split_geom[scheme == kSchemeStrang];
+}
+
 // The fused split step's arguments: its own tiles and partial sums.
 SplitArgs split_args(fk_grid* g, const StepArgs& step) {
   SplitArgs sa{};
   sa.a = step;
-  sa.a.geom = g->split_geom[g->scheme == kSchemeStrang];
+  sa.a.geom = split_plan(g, g->scheme);
   const int nt = sa.a.geom.n_tiles;
   const size_t np = (size_t)g->nx * nt;
   double* b = g->d_split_part;
@@ -319,7 +324,7 @@ cudaError_t enqueue_step(fk_grid* g, int cur, cudaStream_t s, cudaEvent_t ev0, c
   cudaError_t e = cudaSuccess;
   if (ev0) e = cudaEventRecord(ev0, s);
   if (e == cudaSuccess) {
-    if (g->scheme != kSchemeUnsplit && g->split_geom[0].n_tiles > 0) {
+    if (g->scheme != kSchemeUnsplit && split_plan(g, g->scheme).n_tiles > 0) {
       const SplitArgs sa = split_args(g, a);
       e = launch_split_step(sa, g->prec, g->scheme == kSchemeStrang, g->prm.collisions != 0, s);
       a.part = sa.a.part;  // what the finalize folds
@@ -502,8 +507,9 @@ cudaError_t dalloc(P** p, size_t bytes) {
 // steps: their partial sums and boundary planes.  Split steps as passes: a
 // third buffer of f, and the Strang step's second state block.
 fk_status split_buffers(fk_grid* g, int scheme) {
-  if (scheme != kSchemeUnsplit && g->split_geom[0].n_tiles > 0) {
-    const size_t n = (2 * (size_t)g->nx + 6) * g->split_geom[0].n_tiles * sizeof(double);
+  if (scheme != kSchemeUnsplit && split_plan(g, scheme).n_tiles > 0) {
+    // (both schemes' plans have the same tiles)
+    const size_t n = (2 * (size_t)g->nx + 6) * split_plan(g, scheme).n_tiles * sizeof(double);
     if (!g->d_split_part) {
       FK_CUDA(g, dalloc(&g->d_split_part, n));
       FK_CUDA(g, cudaMemsetAsync(g->d_split_part, 0, n, g->stream));
@@ -648,12 +654,10 @@ fk_status plan_geometry(fk_grid* g) {
     }
   }
   plan_resident(g, sms);
-  Geom sg[2]{};
-  if (g->use_stream && plan_split(g->prec, false, g->nx, g->nv1, g->pitch, i_neg, sms, &sg[0]) &&
-      plan_split(g->prec, true, g->nx, g->nv1, g->pitch, i_neg, sms, &sg[1])) {
-    g->split_geom[0] = sg[0];
-    g->split_geom[1] = sg[1];
-  }
+  for (int strang = 0; strang < 2 && g->use_stream; strang++)
+    if (!plan_split(g->prec, strang != 0, g->nx, g->nv1, g->pitch, i_neg, m.half != 0, sms,
+                    &g->split_geom[strang]))
+      g->split_geom[strang] = Geom{};
   return FK_OK;
 }
 

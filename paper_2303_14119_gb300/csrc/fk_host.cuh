@@ -88,8 +88,8 @@ struct fk_grid {
   // refused and the getters wait for the batch's last enqueued step
   int scheme = 0;             // kSchemeUnsplit, kSchemeLie or kSchemeStrang
   // the fused split steps (fk_split.cu): the tiles of a Lie and of a Strang
-  // step (none: the steps run as passes; the two differ in their chunks
-  // only), their partial sums in one buffer and the boundary planes of the
+  // step (none: that scheme runs as passes; where both have them they differ
+  // in their chunks only), their partial sums in one buffer and the boundary planes of the
   // state after the velocity step
   fk::Geom split_geom[2]{};
   double* d_split_part = nullptr;

@@ -687,10 +687,31 @@ cudaError_t launch_typed(const SplitArgs& sa, bool strang, bool bgk, cudaStream_
   return cudaGetLastError();
 }
 
+// Whether one march is faster than the passes.  Its planes are a chain of two
+// phases each, which the passes' pipeline of planes has not, so it loses where
+// a chunk has many planes and a plane little work or twice the reads:
+//  - tiles of two rows, whose halo rows double the reads (us a step, march and
+//    passes: Lie FP32 64 x 64 x 2000, 17 planes a chunk, 54 and 56; 256 x 64 x
+//    2000, 65 planes, 157 and 119; FP64 64 x 64 x 1000, 17 planes, 130 and 115,
+//    16 x 32 x 1000, 2 planes, 32 and 58; Strang FP64 64 x 64 x 1000 166 and
+//    168, 256 x 64 x 1000, 65 planes, 536 and 477; Strang FP32 256 x 64 x 2000
+//    169 and 187);
+//  - thin grids, whose passes run as half units (Lie FP32 1024 x 16 x 16, 5
+//    planes, 24.3 and 26.9; 2048 x 16 x 16, 9 planes, 32.9 and 31.5; 8192 x 16 x
+//    16, 36 planes, 87 and 72; FP64, bound by its pipe sooner: 2048 x 32 x 32, a
+//    vector a thread, 61 and 69; 2048 x 8 x 8 60 and 45).
+bool march_pays(bool f32, bool strang, bool half, int most_rows, int vectors, int planes) {
+  if (most_rows == 2) return strang ? f32 || planes <= 16 : planes <= (f32 ? 17 : 6);
+  if (!half) return true;
+  if (f32) return planes <= (vectors < 128 ? 8 : strang ? 14 : 9);
+  if (vectors >= (strang ? 128 : 256)) return true;
+  return planes <= (strang || vectors >= 64 ? 8 : 4);
+}
+
 }  // namespace
 
-bool plan_split(int precision, bool strang, int nx, int nv1, int pitch, int i_neg, int sms,
-                Geom* gm) {
+bool plan_split(int precision, bool strang, int nx, int nv1, int pitch, int i_neg, bool half,
+                int sms, Geom* gm) {
   const int vec = precision == FK_F32 ? 4 : 2;
   const int most = std::min(kSplitThreads * kSplitVec * vec / pitch, kMaxTileRows);
   if (most < 2) return false;  // the halo rows would double the reads
@@ -716,7 +737,8 @@ bool plan_split(int precision, bool strang, int nx, int nv1, int pitch, int i_ne
   m.chunk_len = (nx + last + nc - 1) / nc;
   m.n_chunks = (nx + m.chunk_len - 1) / m.chunk_len;
   *gm = m;
-  return true;
+  return march_pays(precision == FK_F32, strang, half, most,
+                    std::max(m.ti_neg, m.ti_pos) * (pitch / vec), m.chunk_len);
 }
 
 cudaError_t launch_split_step(const SplitArgs& sa, int precision, bool strang, bool bgk,

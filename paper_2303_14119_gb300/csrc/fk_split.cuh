@@ -16,9 +16,10 @@ struct SplitArgs {
 };
 
 // Tiles and chunks of a fused split step for these sizes; false if a plan
-// does not fit (rows too wide for a tile of two of them).
-bool plan_split(int precision, bool strang, int nx, int nv1, int pitch, int i_neg, int sms,
-                Geom* gm);
+// does not fit (rows too wide for a tile of two of them) or the passes are
+// faster.  half: the grid's streaming units are half units.
+bool plan_split(int precision, bool strang, int nx, int nv1, int pitch, int i_neg, bool half,
+                int sms, Geom* gm);
 // One Lie (strang = false) or Strang step of f_in into f_out, without its
 // finalize; the second also adds the mid-step fluxes' share to a.st.
 cudaError_t launch_split_step(const SplitArgs& sa, int precision, bool strang, bool bgk,

@@ -5,6 +5,8 @@ either sign, and rows too wide for it (the steps then run as passes).
 
 Bounds: one step's rounding of FP64 and FP32, those of the tests of the
 passes; sums over a plane take the same."""
+import time
+
 import numpy as np
 import pytest
 
@@ -61,3 +63,34 @@ def test_withheld_copy_times_out_and_the_state_stays(scheme, item, monkeypatch):
         g.get_f(out)
     assert np.array_equal(out, start)
     g.close()
+
+
+# either side of the line between one march and the passes: tiles of two rows,
+# thin grids of a few and of many planes per chunk
+@pytest.mark.parametrize("scheme", [fk.FK_SCHEME_LIE, fk.FK_SCHEME_STRANG])
+@pytest.mark.parametrize("prec,tol", [(fk.FK_F64, 1e-12), (fk.FK_F32, 5e-7)])
+@pytest.mark.parametrize("shape", [(40, 8, 1800), (300, 6, 1800), (100, 8, 1000), (1030, 8, 8), (2100, 8, 8),
+                                   (2100, 24, 10), (2500, 30, 32)])
+def test_split_steps_on_either_side_of_the_march_rule(shape, prec, tol, scheme):
+    test_split_steps_match_the_oracle(shape, prec, tol, scheme)
+
+
+def test_long_chains_of_little_work_run_as_passes():
+    """An FP64 Lie step of 8192 planes of 8 x 8 against single launches of the
+    unsplit step: two passes take about 1.5 times as long, the march 2.3 times."""
+    times = {}
+    for scheme in (fk.FK_SCHEME_UNSPLIT, fk.FK_SCHEME_LIE):
+        g = fk.Grid(8192, 8, 8, 20e-6, -6e7, 6e7, -3e7, 3e7, cfl=0.4, precision=fk.FK_F64)
+        g.set_fields(-1e5, False, 0.0)
+        g.set_scheme(scheme)
+        g.set_f(np.full((8192, 8, 8), 1e5))
+        g.set_kernel_timing(scheme == fk.FK_SCHEME_UNSPLIT)
+        best = float("inf")
+        for _ in range(6):
+            t = time.perf_counter()
+            g.step(128)
+            g.sync()
+            best = min(best, time.perf_counter() - t)
+        times[scheme] = best
+        g.close()
+    assert times[fk.FK_SCHEME_LIE] < 1.9 * times[fk.FK_SCHEME_UNSPLIT]
