@@ -15,6 +15,7 @@
 namespace {
 
 constexpr int kUnits = 16;  // most partial sums per x-plane
+constexpr int kTwoBlocksPerSm = 2 * 152;  // on GB300
 
 // Scratch shared by every call: FK_NOALLOC_MAX_PARTIALS doubles (1 MiB).
 static __device__ __align__(256) double g_noalloc_partials[FK_NOALLOC_MAX_PARTIALS];
@@ -132,12 +133,19 @@ extern "C" fk_status fk_density_moment_noalloc(const double* f_dev, int32_t nx, 
   }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const long long plane = (long long)nv1 * nv2;
-  // One block a plane wherever there are 64 planes: the second launch costs more
-  // (4 us) than the idle SMs (64 planes of 200 x 200 take 10 us either way, 32 of
-  // 256 x 256 16.5 us whole and 12.3 in slices).  512 threads where they have
-  // more than two groups of values each (1024 planes of 256 x 256: 83 against
-  // 92 us), else 256 (669 planes of 112 x 129: 16 against 18 us).
-  const int units = nx >= 64 ? 1 : std::min(kUnits, (304 + nx - 1) / nx);
+  // One block a plane where the second launch (4 us) costs more than the idle SMs:
+  // from 64 planes on (64 of 200 x 200 take 10 us either way, 32 of 256 x 256
+  // 16.5 us whole and 12.3 in slices), and for small planes (16 of 64 x 64: 4.5
+  // against 10.4 us; 2 of 256 x 256: 12.6 against 8.8).  Large planes that leave
+  // SMs idle are worth the launch (64 of 512 x 512: 48 whole, 29 in four slices;
+  // 64 of 1024 x 1024: 166 and 87; 300 of 512 x 512: the same).  512 threads
+  // where they have more than two groups of values each (1024 planes of 256 x
+  // 256: 83 against 92 us), else 256 (669 planes of 112 x 129: 16 against 18 us).
+  int units = std::min(kUnits, (kTwoBlocksPerSm + nx - 1) / nx);
+  if (plane <= 128 * 128)
+    units = 1;
+  else if (nx >= 64)
+    units = plane >= 512 * 512 && nx < kTwoBlocksPerSm ? 4 : 1;
   const double dvv = dv1 * dv2;
   if (plane / units >= 2 * 512 * fk::kGroup)
     moment_partials<512><<<nx * units, 512, 0, s>>>(f_dev, plane, units, scratch, dvv, n_e_dev);

@@ -60,3 +60,39 @@ def test_negative_and_non_finite_values(torch):
     got = moment(torch, f)
     assert got[0] == 72.0 and got[1] == 66.0 and got[4] == 0.0 and got[5] == 71.0
     assert np.isposinf(got[2]) and np.isnan(got[3]) and np.all(got[6:] == 72.0)
+
+
+# small planes whole and larger ones in slices below 64 planes, large planes in four
+@pytest.mark.parametrize("shape", [(2, 128, 128), (2, 113, 146), (64, 512, 512), (65, 513, 513),
+                                   (303, 512, 512), (304, 512, 512)])
+def test_sums_on_either_side_of_the_slicing_rule(torch, shape):
+    gen = torch.Generator(device="cuda").manual_seed(shape[0])
+    f = torch.rand(shape, generator=gen, dtype=torch.float64, device="cuda")
+    n_e = torch.empty(shape[0], dtype=torch.float64, device="cuda")
+    fk.fk_density_moment_noalloc(f.data_ptr(), *shape, 1.0, 1.0, n_e.data_ptr(),
+                                 torch.cuda.current_stream().cuda_stream or None)
+    # multiples of 2^-53 below 1: whole sums below 2^64 as two halves
+    hi = torch.floor(f * 2.0 ** 26).to(torch.int64)
+    lo = (f * 2.0 ** 26 - hi) * 2.0 ** 27
+    ref = (hi.sum((1, 2)).double() + lo.to(torch.int64).sum((1, 2)).double() * 2.0 ** -27) * 2.0 ** -26
+    assert ((n_e - ref).abs() <= 1e-15 * ref).all()
+
+
+def test_few_large_planes_take_no_longer_than_many_small_ones(torch):
+    """The same 0.5 GB as 64 planes and as 1024: 87 and 82 us (166 with 64 blocks
+    on 152 SMs)."""
+    def best(shape):
+        f = torch.rand(shape, dtype=torch.float64, device="cuda")
+        n_e = torch.empty(shape[0], dtype=torch.float64, device="cuda")
+        times = []
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(10):
+                fk.fk_density_moment_noalloc(f.data_ptr(), *shape, 1.0, 1.0, n_e.data_ptr(),
+                                             torch.cuda.current_stream().cuda_stream or None)
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1))
+        return min(times)
+    assert best((64, 1024, 1024)) < 1.5 * best((1024, 256, 256))
