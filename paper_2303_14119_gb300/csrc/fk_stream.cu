@@ -73,6 +73,16 @@ step_stream_batch_half_kernel(const BatchInst* __restrict__ inst, const int4* __
   stream_unit<T, PADDED, BGK, kHalfThreads, true>(a, u % nt, u / nt, region + kArgsBytes, ht, 1 + h);
 }
 
+// FP32 grids with collisions take the kernel for padded rows, whose rows may
+// also have no padding: the compiler keeps it within its registers, the other
+// one spilled 32 bytes in its march (batches of unpadded grids, us a step: four
+// of 1024 x 128 x 128 150 -> 132, three of 512 x 256 x 256 200 -> 179, twelve of
+// a sweep 127 -> 112; before the two-cell update 147, 191 and 124).
+template <typename T, bool PADDED, bool BGK>
+constexpr auto batch_kernel() {
+  return step_stream_batch_kernel<T, PADDED || (BGK && sizeof(T) == 4), BGK>;
+}
+
 }  // namespace
 
 int stream_tile_rows(int precision, int pitch, int smem_per_sm, int reserved_per_block,
@@ -134,7 +144,7 @@ cudaError_t fit_kernel(K k, int optin, size_t smem_bytes, bool count, int* best)
 template <typename T, bool P, bool B>
 cudaError_t fit_four(int optin, size_t smem_bytes, bool whole, bool half, int* best) {
   cudaError_t e = fit_kernel(step_stream_kernel<T, P, B>, optin, smem_bytes, whole, best);
-  if (e == cudaSuccess) e = fit_kernel(step_stream_batch_kernel<T, P, B>, optin, smem_bytes, whole, best);
+  if (e == cudaSuccess) e = fit_kernel(batch_kernel<T, P, B>(), optin, smem_bytes, whole, best);
   if (e == cudaSuccess) e = fit_kernel(step_stream_half_kernel<T, P, B>, optin, smem_bytes, half, best);
   if (e == cudaSuccess)
     e = fit_kernel(step_stream_batch_half_kernel<T, P, B>, optin, smem_bytes, half, best);
@@ -188,9 +198,9 @@ void launch_batch(const BatchInst* inst, const int2* units, int n_units, size_t 
                   const int4* pairs, int n_pairs, int half_bytes, bool padded, cudaStream_t s) {
   if (n_units > 0) {
     if (padded)
-      step_stream_batch_kernel<T, true, BGK><<<n_units, kBlock, smem, s>>>(inst, units);
+      batch_kernel<T, true, BGK>()<<<n_units, kBlock, smem, s>>>(inst, units);
     else
-      step_stream_batch_kernel<T, false, BGK><<<n_units, kBlock, smem, s>>>(inst, units);
+      batch_kernel<T, false, BGK>()<<<n_units, kBlock, smem, s>>>(inst, units);
   }
   if (n_pairs > 0) {
     const size_t hs = 2 * (size_t)half_bytes;

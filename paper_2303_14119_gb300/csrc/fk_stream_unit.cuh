@@ -527,9 +527,11 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
   constexpr int VEC = Vec<T>::N;
   constexpr int M = unit_vectors<NT, (int)sizeof(T)>();
   // per-plane pointer reads from the shared-memory arguments at their use
-  // where the march runs out of registers (half units, the collision
-  // variant); elsewhere the pointers stay in registers (measured faster)
-  constexpr bool SAU = SA && (NT == kHalfThreads || BGK);
+  // where the march runs out of registers (half units, FP64 grids with
+  // collisions); elsewhere the pointers stay in registers (measured faster;
+  // FP32 batches with collisions spilled 20 bytes with them read at use and
+  // none without: four grids of 1024 x 128 x 128 139 -> 132 us a step)
+  constexpr bool SAU = SA && (NT == kHalfThreads || (BGK && sizeof(T) == 8));
   // compact index arithmetic (an item's plane in one multiply-add, 32-bit
   // stage and plane sizes), where it keeps the march's registers within the
   // launch bounds: without it the plain whole-CTA FP32 batch kernel spills 40

@@ -209,3 +209,21 @@ def test_lie_multi_step_ledger_and_switching_back():
     o.step(33)
     assert rel_l1(g.get_f(), o.get_f()) <= 1e-10
     g.close()
+
+
+@pytest.mark.parametrize("shapes", [[(9, 96, 64), (30, 117, 128)], [(9, 96, 64), (21, 70, 93)]])
+def test_whole_cta_batch_with_collisions_bitwise(shapes):
+    """FP32 grids whose units take a CTA each, rows without padding alone and
+    beside rows with it: one kernel steps both, as the grids alone."""
+    grids = [[setup(s, fk.FK_F32, 60 + q, dtnu=0.02)[0] for q, s in enumerate(shapes)]
+             for _ in range(2)]
+    with fk.Batch(grids[1]) as b:
+        b.step(33)
+        assert b.sync() == [fk.FK_OK] * len(shapes)
+    for ga, gb in zip(*grids):
+        ga.step(33)
+        assert np.array_equal(ga.get_f(), gb.get_f())
+        assert ga.surface_charge() == gb.surface_charge()
+        assert ga.ledger() == gb.ledger()
+        ga.close()
+        gb.close()
