@@ -208,10 +208,10 @@ def make_grids(fk, w, precision, stream, phys=None):
 def time_arm(fk, torch, w, precision, f0, steps, warmup, dist, device, batch=True,
              kernel_steps=50, chunk_len=0, tile_rows=-1, phys=None):
     """Time `steps` steps of the workload's instances after `warmup` steps,
-    as users run them: each step a CUDA-graph replay (batch: one step-kernel
-    launch per unit layout and one finalize launch for all instances, x-chunks
-    and v1 tiles autotuned before the warm-up; else each instance's own
-    graph).  chunk_len > 0 pins the x-chunks, tile_rows >= 0 the tile-row cap
+    as users run them: as a batch, CUDA-graph replays (one step-kernel launch
+    per unit layout and one finalize launch a step for all instances, x-chunks
+    and v1 tiles autotuned before the warm-up); else fk_step(1) of one instance
+    after another (an unsplit step on streaming tiles: one resident launch).  chunk_len > 0 pins the x-chunks, tile_rows >= 0 the tile-row cap
     (0: the default tiles), each instead of the autotuner's choice.  The
     step kernel's own launch durations (CUDA events around each launch,
     direct launches) are taken in a separate pass of `kernel_steps` steps
@@ -300,14 +300,20 @@ def time_arm(fk, torch, w, precision, f0, steps, warmup, dist, device, batch=Tru
             g.set_kernel_timing(False)
             g.sync()
         info = grids[0].info()
-        plan = dict(mode="per-instance", timed="CUDA-graph replay per instance",
+        scheme = phys["scheme"] if phys else "unsplit"
+        resident = scheme == "unsplit" and info["kernel"] == "stream"
+        # split steps: the march, the Strang step's x = 0 plane, the finalize
+        # (the fewest: grids whose rule takes the passes launch more)
+        per_step = 1 if resident else {"unsplit": 2, "lie": 2, "strang": 3}[scheme]
+        plan = dict(mode="per-instance",
+                    timed="fk_step(1) of one instance after another: " +
+                          ("a resident launch each" if resident else "%d launches each" % per_step),
+                    kernel_times="CUDA events around each step's kernels, separate pass of %d "
+                                 "steps%s" % (kernel_steps, " in single launches, whose tiles and "
+                                              "chunks these are" if resident else ""),
                     **{k: info[k] for k in ("kernel", "n_tiles", "n_chunks", "chunk_len")})
         cells_per_launch = cells
-        # split steps: the march, the Strang step's x = 0 plane, the finalize;
-        # unsplit steps of one grid: up to 128 in a launch
-        scheme = phys["scheme"] if phys else "unsplit"
-        per_grid = {"unsplit": -(-steps // 128), "lie": 2 * steps, "strang": 3 * steps}[scheme]
-        gpu_launches = per_grid * len(grids)
+        gpu_launches = per_step * steps * len(grids)
     return dict(ms=ms, launches=launches, kernel_ms=kms, cells=cells, n_inst=len(grids),
                 cells_per_launch=cells_per_launch, gpu_launches=gpu_launches, clocks=ck,
                 grids=grids, kernel=plan)
@@ -511,7 +517,7 @@ def run_ours(args):
         line["config"]["physics"] = dict(
             collisions="BGK, T_e 2 eV, ln Lambda 10" if args.collisions else "off",
             reflection=args.reflection, scheme=args.scheme,
-            passes_per_step=1, timed_launches="the step kernel")
+            timed_launches="one step's kernels without its finalize")
     if not args.no_side:
         other = "f64" if args.precision == "f32" else "f32"
         oprec = fk.FK_F64 if other == "f64" else fk.FK_F32
@@ -569,7 +575,7 @@ def measure_sweep(fk, torch, workload, precision, steps, warmup, dist, local, wo
     (synth.sweep_instances) or of the surrogate's training runs
     (synth.surrogate_runs) stepped as one batch (x-chunks autotuned per size
     bucket), against the same instances stepped one after another with
-    fk_step (each instance's steps as CUDA-graph replays).  Both arms give
+    fk_step (each instance's steps in resident launches).  Both arms give
     bitwise identical states; the metric is instances per hour at the
     workload's steps per instance, from the timed per-step rate.  Returns
     the JSON object of the measurement."""
