@@ -536,9 +536,11 @@ __device__ __forceinline__ void stream_unit(const StepArgs& a, const int t, cons
   // stage and plane sizes), where it keeps the march's registers within the
   // launch bounds: without it the plain whole-CTA FP32 batch kernel spills 40
   // bytes in the march, and three grids of 1024 x 256 x 256 take 318 us a
-  // launch instead of 263 (0.745 and 0.90 of copy bandwidth).  The FP64 and the
-  // resident plain whole-CTA kernels spill less without it.
-  constexpr bool COMPACT = NT == kHalfThreads || PADDED || BGK || (!RES && sizeof(T) == 4);
+  // launch instead of 263 (0.745 and 0.90 of copy bandwidth).  The other plain
+  // whole-CTA kernels do without: a grid alone has no spill either way (with it
+  // 104 us instead of 99.7 at 1024 x 256 x 256, 49 instead of 52 at 600 x 200 x
+  // 200), the FP64 and the resident ones spill less.
+  constexpr bool COMPACT = NT == kHalfThreads || PADDED || BGK || (SA && sizeof(T) == 4);
   using StageSz = std::conditional_t<COMPACT, unsigned, size_t>;  // < 227 KB
   using PlaneSz = std::conditional_t<COMPACT, int, size_t>;
   const Geom& gm = a.geom;
