@@ -199,11 +199,12 @@ fk_status fk_set_reflection(fk_grid *grid, double R_f);
  * from its own input state, so the surface charge and the wall ledger terms
  * take dt/2 of the fluxes of f^n and dt/2 of those of the state after the
  * velocity step.  Sec. 2 states only an explicit upwind update.  A split step
- * is one pass over f (a kernel of its own); on grids too wide for its tiles it
- * runs as two (Lie) or three (Strang) passes through one more buffer of f,
- * each the streaming step kernel with the other terms' coefficients zeroed
- * (the direct-load kernel on grids too wide for that),
- * and grids using them cannot join a batch.  FK_EINVAL for another value;
+ * is one pass over f (a kernel of its own); on grids too wide for its tiles,
+ * and on thin grids of many planes and rows of more than 1365 FP32 or 682 FP64
+ * cells where that is faster, it runs as two (Lie) or three (Strang) passes
+ * through one more buffer of f, each the streaming step kernel with the other
+ * terms' coefficients zeroed (the direct-load kernel on grids too wide for
+ * that).  Grids using split schemes cannot join a batch.  FK_EINVAL for another value;
  * FK_ESTATE while the grid is in a batch. */
 #define FK_SCHEME_UNSPLIT 0
 #define FK_SCHEME_LIE 1
@@ -218,8 +219,11 @@ fk_status fk_set_convergence(fk_grid *grid, int64_t window, double rel_tol);
 
 /* Advance n >= 0 time steps (forward Euler, all fluxes from f^n; Eq. 18
  * updates sigma for the next step's E_x).  Stream-ordered and asynchronous:
- * it returns once the work is enqueued.  Returns a sticky device error seen
- * by an earlier synchronising call (FK_ECFL, FK_ENUMERIC, FK_ETIMEOUT). */
+ * it returns once the work is enqueued.  Unsplit steps of a streaming grid run
+ * up to 128 to a cooperative launch, or each in launches of its own while grids
+ * or batches on other streams are stepped at the same time and the GPU cannot
+ * hold the CTAs of all; both give the same bits.  Returns a sticky device error
+ * seen by an earlier synchronising call (FK_ECFL, FK_ENUMERIC, FK_ETIMEOUT). */
 fk_status fk_step(fk_grid *grid, int64_t n);
 
 /* Wait for the grid's stream and report any sticky device error. */
@@ -308,9 +312,9 @@ fk_status fk_grid_info(const fk_grid *grid, double *out);
 fk_status fk_set_tile_rows(fk_grid *grid, int32_t max_rows);
 
 /* Kernel timing (tracing).  enabled != 0: later fk_step calls launch each
- * step directly (no graph replay) and record a CUDA event pair around every
- * launch of the fused step kernel on the grid's stream; enabled = 0 returns
- * to graph replay.  Switching discards pending records. */
+ * step directly (no resident launch, no graph replay) and record a CUDA event
+ * pair around every launch of the fused step kernel on the grid's stream;
+ * enabled = 0 returns to them.  Switching discards pending records. */
 fk_status fk_set_kernel_timing(fk_grid *grid, int enabled);
 
 /* Synchronise and report the step-kernel launches recorded since the last

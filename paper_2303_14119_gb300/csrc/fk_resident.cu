@@ -22,18 +22,22 @@
 //
 // What bounds it: on small grids the chain arrival -> partial sums -> scan ->
 // E_x -> go (about 3.5 us on one finalize CTA, 5 us on several) and the unit
-// that holds the wall; on large ones HBM.  Measured, us a step, two launches
-// a step replayed as graphs -> here: 64 x 48 x 48 FP64 34.7 -> 16.1, FP32 21.8
-// -> 9.8; 321 x 117 x 117 FP32 25.9 -> 21.6; 512 x 128 x 128 FP32 with
-// collisions 32.9 -> 24.1; 1024 x 256 x 256 FP32 109.8 -> 101.4, FP64 622 -> 574.
+// that holds the wall; on large ones HBM (FP32) or the FP64 pipe.  Measured, us
+// a step, two launches a step replayed as graphs -> here: 64 x 48 x 48 FP64 34.9
+// -> 15.4, FP32 20.4 -> 10.4; 321 x 117 x 117 FP32 26.2 -> 21.6; 512 x 128 x 128
+// FP32 with collisions and reflection 33.0 -> 26.2; 1024 x 256 x 256 FP32 109.7
+// -> 105.3, FP64 620 -> 576.  (The FP32 kernels of whole-CTA units spill 52 to
+// 116 bytes; the two-launch step kernel of the largest grid takes 99.7 us of its
+// 109.7 without a spill.)
 //
 // Waits: every block of the launch is resident (cooperative launch), every
 // wait is bounded by Params::wait_limit, and after one that runs out the
-// launch ends with kFlagTimeout set and the state of the last whole step.
+// launch ends with kFlagTimeout set and the state of the last whole step.  A
+// finalize CTA that finds a Courant or non-finite fault in the new state ends
+// the launch after that step, through both counters (kGoStop).
 #include <stddef.h>
 
 #include <algorithm>
-
 
 #include "fk_finalize.cuh"
 #include "fk_resident.cuh"
